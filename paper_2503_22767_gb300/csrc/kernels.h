@@ -28,7 +28,12 @@ struct StepArgs {
     float* gmag = nullptr;
     const float* field = nullptr;    // [inst][n_steps][D]
     float* gfield = nullptr;
-    float* mom = nullptr;            // [n_steps][n_inst] sum_p m_p v_x after each substep
+    // sum_p m_p v_x after each substep: the forward adds in 64 bits to
+    // [n_steps][n_inst][mom_slots] (mom_acc; warp w adds to slot w % mom_slots,
+    // a power of two), the adjoint reads the finished rows [n_steps][n_inst]
+    double* mom_acc = nullptr;
+    int mom_slots = 1;
+    const float* mom = nullptr;
     const float* Minst = nullptr;    // [n_inst] instance mass
     const float* dloss = nullptr;    // [n_inst]
     const int* inst_off = nullptr;   // [n_inst + 1]
@@ -123,11 +128,13 @@ cudaError_t launch_scatter_design_grad(int dim, const Params& P, const int* id,
                                        const float* gmag, long long nd, float* g_phi,
                                        float* g_mag, cudaStream_t st);
 cudaError_t launch_instance_mass(const Params& P, const float* phi, const int* inst_off,
-                                 float* Minst, cudaStream_t st);
-// (x0: current-order initial positions; the state holds displacements)
+                                 double* mass_acc, cudaStream_t st);
+// The objective of every instance.  (x0: current-order initial positions; the
+// state holds displacements.)  Locomotion: also the finished momentum rows
+// mom [n_steps][n_inst] and instance masses Minst from the 64-bit sums.
 cudaError_t launch_loss(int dim, const Params& P, const float* s, const float* x0, const float* target,
-                        const int* id, const int* inst_off, const float* Minst, const float* mom,
-                        float* loss_acc, float* loss_out, cudaStream_t st);
+                        const int* id, const int* inst_off, const double* mass_acc, const double* mom_acc,
+                        int mom_slots, double* loss_acc, float* Minst, float* mom, float* loss_out, cudaStream_t st);
 cudaError_t launch_seed(int dim, const Params& P, const float* s, const float* x0, const float* target,
                         const int* id, const int* inst_off, const float* phi, const float* Minst,
                         const float* mom, const float* dloss, float* adj, float* gphi,

@@ -197,18 +197,18 @@ __global__ void k_scatter_design_grad(Params P, const int* __restrict__ id,
 }
 
 __global__ void k_instance_mass(Params P, const float* __restrict__ phi,
-                                const int* __restrict__ inst_off, float* __restrict__ Minst) {
+                                const int* __restrict__ inst_off, double* __restrict__ mass_acc) {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     bool active = p < P.n_total;
     int inst = active ? find_instance(inst_off, P.n_inst, p) : -1;
     float m[1] = {active ? phi[p] * P.rho0 * P.p_vol : 0.0f};
-    warp_add_per_instance<1>(m, inst, Minst, 1);
+    warp_add_per_instance<1>(m, inst, mass_acc, 1);
 }
 
 template <int D>
 __global__ void k_loss_mse(Params P, const float* __restrict__ s, const float* __restrict__ x0,
                            const float* __restrict__ target, const int* __restrict__ id,
-                           const int* __restrict__ inst_off, float* __restrict__ loss_acc) {
+                           const int* __restrict__ inst_off, double* __restrict__ loss_acc) {
     using L = Layout<D>;
     int p = blockIdx.x * blockDim.x + threadIdx.x;
     bool active = p < P.n_total;
@@ -226,19 +226,38 @@ __global__ void k_loss_mse(Params P, const float* __restrict__ s, const float* _
     warp_add_per_instance<1>(e2, inst, loss_acc, 1);
 }
 
-__global__ void k_loss_finalize(Params P, const int* __restrict__ inst_off,
-                                const float* __restrict__ Minst, const float* __restrict__ mom,
-                                const float* __restrict__ loss_acc, float* __restrict__ loss_out) {
-    int inst = blockIdx.x * blockDim.x + threadIdx.x;
-    if (inst >= P.n_inst) return;
-    if (P.loss_kind == 1) {
-        float M = Minst[inst];
-        double acc = 0.0;
-        for (int n = 0; n < P.n_steps; ++n) acc += mom[(long long)n * P.n_inst + inst];
-        loss_out[inst] = M > 0.0f ? (float)(-(double)P.dt * acc / M) : 0.0f;
-    } else {
-        int cnt = inst_off[inst + 1] - inst_off[inst];
-        loss_out[inst] = cnt > 0 ? loss_acc[inst] / (float)cnt : 0.0f;
+// One block per instance: its threads share the substeps (a single thread
+// walking 5,000 rows is a chain of 5,000 dependent additions and loads).
+constexpr int kFinalizeThreads = 256;
+
+__global__ void __launch_bounds__(kFinalizeThreads)
+    k_loss_finalize(Params P, const int* __restrict__ inst_off, const double* __restrict__ mass_acc,
+                    const double* __restrict__ mom_acc, int mom_slots, const double* __restrict__ loss_acc,
+                    float* __restrict__ Minst, float* __restrict__ mom, float* __restrict__ loss_out) {
+    const int inst = blockIdx.x;
+    if (P.loss_kind != 1) {
+        const int cnt = inst_off[inst + 1] - inst_off[inst];
+        if (threadIdx.x == 0) loss_out[inst] = cnt > 0 ? (float)(loss_acc[inst] / cnt) : 0.0f;
+        return;
+    }
+    __shared__ double part[kFinalizeThreads];
+    double acc = 0.0;
+    for (int n = threadIdx.x; n < P.n_steps; n += kFinalizeThreads) {
+        const double* slots = mom_acc + ((long long)n * P.n_inst + inst) * mom_slots;
+        double row = 0.0;
+        for (int k = 0; k < mom_slots; ++k) row += slots[k];
+        mom[(long long)n * P.n_inst + inst] = (float)row;
+        acc += row;
+    }
+    part[threadIdx.x] = acc;
+    for (int half = kFinalizeThreads / 2; half > 0; half >>= 1) {
+        __syncthreads();
+        if (threadIdx.x < half) part[threadIdx.x] += part[threadIdx.x + half];
+    }
+    if (threadIdx.x == 0) {
+        const double M = mass_acc[inst];
+        Minst[inst] = (float)M;
+        loss_out[inst] = (float)M > 0.0f ? (float)(-(double)P.dt * part[0] / M) : 0.0f;
     }
 }
 
@@ -391,21 +410,22 @@ cudaError_t launch_scatter_design_grad(int dim, const Params& P, const int* id,
 }
 
 cudaError_t launch_instance_mass(const Params& P, const float* phi, const int* inst_off,
-                                 float* Minst, cudaStream_t st) {
+                                 double* mass_acc, cudaStream_t st) {
     if (P.n_total == 0) return cudaSuccess;
-    k_instance_mass<<<blocks_for(P.n_total, 256), 256, 0, st>>>(P, phi, inst_off, Minst);
+    k_instance_mass<<<blocks_for(P.n_total, 256), 256, 0, st>>>(P, phi, inst_off, mass_acc);
     return cudaGetLastError();
 }
 
 cudaError_t launch_loss(int dim, const Params& P, const float* s, const float* x0, const float* target,
-                        const int* id, const int* inst_off, const float* Minst, const float* mom,
-                        float* loss_acc, float* loss_out, cudaStream_t st) {
+                        const int* id, const int* inst_off, const double* mass_acc, const double* mom_acc,
+                        int mom_slots, double* loss_acc, float* Minst, float* mom, float* loss_out, cudaStream_t st) {
     if (P.loss_kind == 0 && P.n_total > 0) {
         dim3 grid(blocks_for(P.n_total, 256));
         if (dim == 2) k_loss_mse<2><<<grid, 256, 0, st>>>(P, s, x0, target, id, inst_off, loss_acc);
         else k_loss_mse<3><<<grid, 256, 0, st>>>(P, s, x0, target, id, inst_off, loss_acc);
     }
-    k_loss_finalize<<<blocks_for(P.n_inst, 64), 64, 0, st>>>(P, inst_off, Minst, mom, loss_acc, loss_out);
+    k_loss_finalize<<<P.n_inst, kFinalizeThreads, 0, st>>>(P, inst_off, mass_acc, mom_acc, mom_slots, loss_acc, Minst, mom,
+                                                          loss_out);
     return cudaGetLastError();
 }
 

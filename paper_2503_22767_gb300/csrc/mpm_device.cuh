@@ -818,9 +818,10 @@ __device__ __forceinline__ void grid_velocity_adjoint(const Params& P, const int
 // Warp-aggregated add of per-lane values into dst[inst * stride + c]: lanes
 // of one instance are summed with shuffles first (the common case), mixed
 // warps fall back to per-lane atomics.  Every lane of the warp must call it.
-template <int NC>
-__device__ __forceinline__ void warp_add_per_instance(const float (&val)[NC], int inst,
-                                                      float* __restrict__ dst, long long stride) {
+// T: float, or double where thousands of warps add to one value.
+template <int NC, typename T>
+__device__ __forceinline__ void warp_add_per_instance(const float (&val)[NC], int inst, T* __restrict__ dst,
+                                                      long long stride) {
     const unsigned full = 0xffffffffu;
     int inst0 = __shfl_sync(full, inst, 0);
     bool uniform = __all_sync(full, inst == inst0 || inst < 0) && inst0 >= 0;
@@ -830,12 +831,12 @@ __device__ __forceinline__ void warp_add_per_instance(const float (&val)[NC], in
             float s = val[c];
 #pragma unroll
             for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(full, s, off);
-            if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(dst + (long long)inst0 * stride + c, s);
+            if ((threadIdx.x & 31) == 0 && s != 0.0f) atomicAdd(dst + (long long)inst0 * stride + c, (T)s);
         }
     } else if (inst >= 0) {
 #pragma unroll
         for (int c = 0; c < NC; ++c)
-            if (val[c] != 0.0f) atomicAdd(dst + (long long)inst * stride + c, val[c]);
+            if (val[c] != 0.0f) atomicAdd(dst + (long long)inst * stride + c, (T)val[c]);
     }
 }
 

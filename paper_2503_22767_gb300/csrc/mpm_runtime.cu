@@ -94,9 +94,12 @@ struct mpm_handle {
     float* mag_d = nullptr;
     float* field = nullptr;
     float* target = nullptr;
-    float* mom = nullptr;
+    float* mom = nullptr;      // momentum rows and masses the adjoint reads (finished by the loss kernel)
     float* Minst = nullptr;
-    float* loss_acc = nullptr;
+    double* mom_acc = nullptr;   // the forward's 64-bit sums: [T][n_inst][mom_slots], [n_inst], [n_inst]
+    double* mass_acc = nullptr;
+    double* loss_acc = nullptr;
+    int mom_slots = 1;
     float* dloss = nullptr;
     float* gphi_d = nullptr;
     float* gmag_d = nullptr;
@@ -603,7 +606,12 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
     ALLOC(h->mag_d, d * h->Nd);
     ALLOC(h->field, (long long)h->n_inst * h->T * d);
     ALLOC(h->target, d * h->N);
+    // a slot of the momentum rows takes the warps of about 2,048 particles:
+    // one for a small body, 16 for a million particles
+    while (h->mom_slots < 16 && (long long)h->mom_slots * 2 * 2048 * h->n_inst <= h->N) h->mom_slots *= 2;
     ALLOC(h->mom, (long long)h->T * h->n_inst);
+    ALLOC(h->mom_acc, (long long)h->T * h->n_inst * h->mom_slots);
+    ALLOC(h->mass_acc, h->n_inst);
     ALLOC(h->Minst, h->n_inst);
     ALLOC(h->loss_acc, h->n_inst);
     ALLOC(h->dloss, h->n_inst);
@@ -785,7 +793,7 @@ int resident_segments(const mpm_handle* h, int n_seg) {
     return std::min(h->n_res, n_seg);
 }
 
-int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStream_t st, float* mom = nullptr);
+int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStream_t st, double* mom_acc = nullptr);
 
 // --- the forward pass: library-owned buffers only, so it can be captured ---
 int forward_pass(mpm_handle* h, cudaStream_t st) {
@@ -798,9 +806,9 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
     auto acc3 = [&](int i) { return h->acc3 + G * (i % 3); };
     int rc;
     MPM_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
-    MPM_CUDA(h, cudaMemsetAsync(h->mom, 0, sizeof(float) * h->T * h->n_inst, st));
-    MPM_CUDA(h, cudaMemsetAsync(h->Minst, 0, sizeof(float) * h->n_inst, st));
-    MPM_CUDA(h, cudaMemsetAsync(h->loss_acc, 0, sizeof(float) * h->n_inst, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->mom_acc, 0, sizeof(double) * h->T * h->n_inst * h->mom_slots, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->mass_acc, 0, sizeof(double) * h->n_inst, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->loss_acc, 0, sizeof(double) * h->n_inst, st));
     if (fuse) MPM_CUDA(h, cudaMemsetAsync(h->acc3, 0, sizeof(float4) * 2 * G, st));
     else MPM_CUDA(h, cudaMemsetAsync(h->acc, 0, sizeof(float4) * G, st));
     // 3D with the grid kernel: the P2G kernels list the node blocks they
@@ -860,9 +868,10 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
         MPM_CUDA(h, cudaMemcpyAsync(h->ck_perm + h->np * seg, h->perm, sizeof(int) * h->np,
                                     cudaMemcpyDeviceToDevice, st));
         StepArgs a = base_args(h);
-        a.mom = h->mom;
+        a.mom_acc = h->mom_acc;
+        a.mom_slots = h->mom_slots;
         if (seg == 0 && (rc = counted(h, 1, [&] {
-                             return mpm::launch_instance_mass(P, h->phi_cur, h->d_inst_off, h->Minst, st);
+                             return mpm::launch_instance_mass(P, h->phi_cur, h->d_inst_off, h->mass_acc, st);
                          })))
             return rc;
         if (seg >= first_res) {
@@ -872,7 +881,7 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
             const int Ks = s1 - s0;
             // lists: the set holds nothing from an earlier forward pass
             if (h->blocks && h->grid_blocks && (rc = clear_list(h, ss.list_id, ss.acc, G, Ks, st))) return rc;
-            if ((rc = recompute_segment(h, seg, T, ss, st, h->mom))) return rc;
+            if ((rc = recompute_segment(h, seg, T, ss, st, h->mom_acc))) return rc;
             MPM_CUDA(h, cudaMemcpyAsync(cur, ss.state + S * Ks, sizeof(float) * S, cudaMemcpyDeviceToDevice, st));
             continue;
         }
@@ -940,8 +949,8 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
         }
     }
     if ((rc = counted(h, 2, [&] {
-             return mpm::launch_loss(d, P, cur, h->x0_fwd, h->target, id_cur, h->d_inst_off, h->Minst, h->mom,
-                                     h->loss_acc, h->st_loss, st);
+             return mpm::launch_loss(d, P, cur, h->x0_fwd, h->target, id_cur, h->d_inst_off, h->mass_acc,
+                                     h->mom_acc, h->mom_slots, h->loss_acc, h->Minst, h->mom, h->st_loss, st);
          })))
         return rc;
     h->cur = cur;
@@ -957,10 +966,10 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
 // so with two streams they overlap: the segment buffers and the
 // current-order design come in two sets, used by segment parity.
 
-// mom: the forward pass's momentum rows (locomotion loss), accumulated by the
+// mom_acc: the forward pass's momentum rows (locomotion loss), accumulated by the
 // G2P of each substep when the forward pass stores a resident segment; null
 // in the backward pass.
-int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStream_t st, float* mom) {
+int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStream_t st, double* mom_acc) {
     const int d = h->dim;
     const Params& P = h->P;
     const long long S = (long long)h->ncomp * h->np;
@@ -1027,7 +1036,8 @@ int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStrea
         a.phi = ss.phi;
         a.mag = ss.mag;
         a.x0 = ss.x0;
-        a.mom = mom;
+        a.mom_acc = mom_acc;
+        a.mom_slots = h->mom_slots;
         a.s_in = state(k);
         a.s_out = state(k + 1);
         a.acc = next_acc;

@@ -200,8 +200,14 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
             }
             mom_x[0] = mp * v[0];
         }
-        if (P.loss_kind == 1 && a.mom != nullptr)
-            warp_add_per_instance<1>(mom_x, inst, a.mom + (long long)a.n_g2p * P.n_inst, 1);
+        // Eq. 40's momentum row: a large body's sum cancels to a small part of
+        // its terms, so thousands of warps add in 64 bits, spread over slots
+        // so that they do not queue for one address
+        if (P.loss_kind == 1 && a.mom_acc != nullptr)
+            warp_add_per_instance<1>(mom_x, inst,
+                                     a.mom_acc + (long long)a.n_g2p * P.n_inst * a.mom_slots +
+                                         ((p >> 5) & (a.mom_slots - 1)),
+                                     a.mom_slots);
     }
     if (P2G) {
         // this warp's box of listed cells, read after the scatter (3D)
