@@ -84,10 +84,12 @@ struct mpm_handle {
     float4* gadj = nullptr;
     float* adj = nullptr;
     float* adj2 = nullptr;
-    float* phi_cur = nullptr;
-    float* mag_cur = nullptr;
-    float* x0_fwd = nullptr;   // forward pass: initial positions in the current order [d][np]
-    float* x0_seg = nullptr;   // recomputation: the same per segment set [2][d][np]
+    float* phi_fwd = nullptr;  // forward pass: design and initial positions in the current order
+    float* mag_fwd = nullptr;
+    float* x0_fwd = nullptr;
+    float* phi_seg = nullptr;  // the same per recomputation set: [2][np], [2][d][np], [2][d][np]
+    float* mag_seg = nullptr;
+    float* x0_seg = nullptr;
     float* gphi_cur = nullptr;
     float* gmag_cur = nullptr;
     float* phi_d = nullptr;
@@ -161,6 +163,18 @@ struct mpm_handle {
     long long spin_limit = 1LL << 22;  // polls before a grid-barrier wait gives up
     unsigned* bar = nullptr;           // grid barrier of the persistent kernels
 
+    // --- stored tail: the two recomputation sets, filled by the forward pass ---
+    // The sets are idle until the backward pass, whose first two recomputed
+    // segments are the last two; so a forward pass that a backward is expected
+    // to follow stores those segments in them as it runs, and the backward
+    // starts with their adjoint.  A store pass costs a forward-only caller 1%
+    // and a clear per substep, so the expectation is that of the last forward:
+    // was it followed by a backward (the design loop), or not (rollouts)?
+    bool last_used = false;    // a backward followed the last forward
+    int n_tail = 0;            // segments of the running pass in the sets (0, 1 or 2)
+    int stored_tail = 0;       // segments the last forward left there, until a backward consumes them
+    bool seg_filled = false;   // 3D lists: the sets hold a forward's segments no adjoint has cleared
+
     // --- options ---
     // grid operation folded into the forward particle kernels (off by default:
     // the autotuner keeps the separate grid kernel on all five workloads)
@@ -174,13 +188,15 @@ struct mpm_handle {
     cudaStream_t aux_stream = nullptr;  // recomputation stream of the backward pass
     cudaEvent_t ev_fork = nullptr, ev_rec[2] = {nullptr, nullptr}, ev_adj[2] = {nullptr, nullptr};
     bool two_streams = true;
-    cudaGraphExec_t exec[2] = {nullptr, nullptr};
-    std::vector<TimedLaunch> graph_timing[2];
+    // each pass has two forms: 0 without and 1 with a stored tail (n_tail)
+    cudaGraphExec_t exec[2][2] = {{nullptr, nullptr}, {nullptr, nullptr}};
+    std::vector<TimedLaunch> graph_timing[2][2];
     bool capturing = false;
-    int capture_pass = 0;
-    long long graph_launches[2] = {0, 0};  // kernels inside each captured graph
-    long long graph_cls[2][4] = {{0, 0, 0, 0}, {0, 0, 0, 0}};  // per kernel class
+    int capture_pass = 0, capture_form = 0;
+    long long graph_launches[2][2] = {{0, 0}, {0, 0}};  // kernels inside each captured graph
+    long long graph_cls[2][2][4] = {};                   // per kernel class
     bool ran_graph[2] = {false, false};
+    int ran_form[2] = {0, 0};
 
     int tune_T = 0;  // > 0 while autotuning: passes stop after this many substeps
 
@@ -235,15 +251,18 @@ int dalloc(mpm_handle* h, T** p, long long count) {
 }
 
 void drop_graphs(mpm_handle* h) {
-    for (int i = 0; i < 2; ++i) {
-        if (h->exec[i]) cudaGraphExecDestroy(h->exec[i]);
-        h->exec[i] = nullptr;
-        for (auto& t : h->graph_timing[i]) {
-            cudaEventDestroy(t.a);
-            cudaEventDestroy(t.b);
+    for (int i = 0; i < 2; ++i)
+        for (int f = 0; f < 2; ++f) {
+            if (h->exec[i][f]) cudaGraphExecDestroy(h->exec[i][f]);
+            h->exec[i][f] = nullptr;
+            for (auto& t : h->graph_timing[i][f]) {
+                cudaEventDestroy(t.a);
+                cudaEventDestroy(t.b);
+            }
+            h->graph_timing[i][f].clear();
         }
-        h->graph_timing[i].clear();
-    }
+    // a changed option may change what a stored segment holds: recompute it
+    h->stored_tail = 0;
 }
 
 // Resident segment sets (MPM_OPT_RESIDENT_SEGMENTS), reserved after creation
@@ -383,7 +402,7 @@ int timed(mpm_handle* h, int cls, double bytes, cudaStream_t st, F&& launch) {
         // event-record nodes of the graph being captured
         MPM_CUDA(h, cudaEventCreate(&ea));
         MPM_CUDA(h, cudaEventCreate(&eb));
-        h->graph_timing[h->capture_pass].push_back(TimedLaunch{cls, ea, eb, bytes});
+        h->graph_timing[h->capture_pass][h->capture_form].push_back(TimedLaunch{cls, ea, eb, bytes});
     } else if (time_it) {
         auto& pool = h->events[cls];
         if (h->ev_used[cls] == pool.size()) {
@@ -424,7 +443,7 @@ int counted(mpm_handle* h, int n, F&& launch) {
 
 // after a stream sync: fold the sampled launches of a replayed graph
 int collect_graph_timing(mpm_handle* h, int pass) {
-    for (auto& t : h->graph_timing[pass]) {
+    for (auto& t : h->graph_timing[pass][h->ran_form[pass]]) {
         float ms = 0.0f;
         MPM_CUDA(h, cudaEventElapsedTime(&ms, t.a, t.b));
         h->timed_ms[t.cls] += ms;
@@ -596,9 +615,11 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
     ALLOC(h->Vbar3, 3 * h->total_nodes);
     ALLOC(h->adj, S);
     ALLOC(h->adj2, S);
-    ALLOC(h->phi_cur, 2 * h->np);
-    ALLOC(h->mag_cur, 2 * d * h->np);
+    ALLOC(h->phi_fwd, h->np);
+    ALLOC(h->mag_fwd, d * h->np);
     ALLOC(h->x0_fwd, d * h->np);
+    ALLOC(h->phi_seg, 2 * h->np);
+    ALLOC(h->mag_seg, 2 * d * h->np);
     ALLOC(h->x0_seg, 2 * d * h->np);
     ALLOC(h->gphi_cur, h->np);
     ALLOC(h->gmag_cur, d * h->np);
@@ -679,8 +700,8 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
 StepArgs base_args(mpm_handle* h) {
     StepArgs a;
     a.x0 = h->x0_fwd;
-    a.phi = h->phi_cur;
-    a.mag = h->mag_cur;
+    a.phi = h->phi_fwd;
+    a.mag = h->mag_fwd;
     a.field = h->field;
     a.inst_off = h->d_inst_off;
     a.err = h->d_err;
@@ -764,8 +785,8 @@ SegSet seg_set(mpm_handle* h, int b) {
     ss.state = h->seg_state + (long long)b * S * (h->K + 1);
     ss.acc = h->seg_acc + (long long)b * G * h->K;
     ss.V = h->seg_V + (long long)b * G * h->K;
-    ss.phi = h->phi_cur + (long long)b * h->np;
-    ss.mag = h->mag_cur + (long long)b * h->dim * h->np;
+    ss.phi = h->phi_seg + (long long)b * h->np;
+    ss.mag = h->mag_seg + (long long)b * h->dim * h->np;
     ss.x0 = h->x0_seg + (long long)b * h->dim * h->np;
     ss.list_id = 2 + b;
     return ss;
@@ -791,6 +812,13 @@ SegSet res_set(mpm_handle* h, int r) {
 int resident_segments(const mpm_handle* h, int n_seg) {
     if (h->tune_T > 0 || use_persist(h)) return 0;
     return std::min(h->n_res, n_seg);
+}
+
+// The segments before the resident ones that the forward pass stores in the
+// recomputation sets (at most two, one per set), if it is asked to.
+int tail_segments(const mpm_handle* h) {
+    if (h->tune_T > 0 || use_persist(h)) return 0;
+    return std::min(2, h->n_seg - resident_segments(h, h->n_seg));
 }
 
 int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStream_t st, double* mom_acc = nullptr);
@@ -828,10 +856,12 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
     int* id_nxt = h->idB;
     const int T = h->tune_T > 0 ? std::min(h->T, h->tune_T) : h->T;
     const int n_seg = (T + h->K - 1) / h->K;
-    // the last n_res segments are stored into resident sets as they run; the
-    // lean substeps end where the first of them begins
+    // the last n_res segments are stored into resident sets as they run, and
+    // the n_tail before them into the recomputation sets; the lean substeps
+    // end where the first of them begins
     const int first_res = n_seg - resident_segments(h, n_seg);
-    const int lean_end = std::min(T, first_res * h->K);
+    const int first_stored = first_res - h->n_tail;
+    const int lean_end = std::min(T, first_stored * h->K);
     if ((rc = counted(h, 1, [&] {
              return mpm::launch_init_state(d, P, h->st_x0, h->st_v0, cur, id_cur, h->x0_fwd, st);
          })))
@@ -857,7 +887,7 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
         }
         if ((rc = counted(h, 1, [&] {
                  return mpm::launch_gather_design(d, P, id_cur, h->d_inst_off, h->d_dbase, h->phi_d,
-                                                  h->mag_d, h->Nd, h->phi_cur, h->mag_cur, h->st_x0,
+                                                  h->mag_d, h->Nd, h->phi_fwd, h->mag_fwd, h->st_x0,
                                                   h->x0_fwd, st);
              })))
             return rc;
@@ -871,13 +901,13 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
         a.mom_acc = h->mom_acc;
         a.mom_slots = h->mom_slots;
         if (seg == 0 && (rc = counted(h, 1, [&] {
-                             return mpm::launch_instance_mass(P, h->phi_cur, h->d_inst_off, h->mass_acc, st);
+                             return mpm::launch_instance_mass(P, h->phi_fwd, h->d_inst_off, h->mass_acc, st);
                          })))
             return rc;
-        if (seg >= first_res) {
-            // a resident segment: every state and grid stored, as a
-            // recomputation would (with the momentum rows of the loss)
-            const SegSet ss = res_set(h, seg - first_res);
+        if (seg >= first_stored) {
+            // a stored segment: every state and grid, as a recomputation
+            // would (with the momentum rows of the loss)
+            const SegSet ss = seg >= first_res ? res_set(h, seg - first_res) : seg_set(h, seg & 1);
             const int Ks = s1 - s0;
             // lists: the set holds nothing from an earlier forward pass
             if (h->blocks && h->grid_blocks && (rc = clear_list(h, ss.list_id, ss.acc, G, Ks, st))) return rc;
@@ -924,7 +954,7 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
                               return mpm::launch_grid(d, P, h->acc, h->V, nullptr, true, n, st);
                           })))
                 return rc;
-            const bool p2g = n + 1 < lean_end;  // a resident segment runs its own first P2G
+            const bool p2g = n + 1 < lean_end;  // a stored segment runs its own first P2G
             const bool all = n + 1 == s1;
             a.s_in = cur;
             a.s_out = nxt;
@@ -1070,7 +1100,10 @@ int finish_adjoint_segment(mpm_handle* h, const int* id_seg, const SegSet& ss, i
                                                     h->gmag_cur, h->Nd, h->gphi_d, h->gmag_d, st);
          })))
         return rc;
-    if (h->blocks && h->grid_blocks && (rc = clear_list(h, ss.list_id, ss.acc, h->total_nodes, Ks, st)))
+    // (a resident set stays as it is: another backward pass may read it, and
+    // the forward pass that refills it empties it first)
+    if (h->blocks && h->grid_blocks && ss.list_id < 4 &&
+        (rc = clear_list(h, ss.list_id, ss.acc, h->total_nodes, Ks, st)))
         return rc;
     return MPM_OK;
 }
@@ -1222,42 +1255,42 @@ int backward_pass(mpm_handle* h, cudaStream_t st) {
     const int n_seg = (T + h->K - 1) / h->K;
     float* adj = h->adj;
     float* adj_next = h->adj2;
-    // segments first_res .. n_seg - 1 were stored by the forward pass
+    // segments first_stored .. n_seg - 1 were stored by the forward pass: in
+    // the resident sets from first_res on, in the recomputation sets before
     const int first_res = n_seg - resident_segments(h, n_seg);
+    const int first_stored = first_res - h->n_tail;
+    auto set_of = [&](int seg) { return seg >= first_res ? res_set(h, seg - first_res) : seg_set(h, seg & 1); };
     // (the persistent kernels each take the whole GPU: one stream)
-    if (!h->two_streams || n_seg < 2 || first_res == 0 || use_persist(h)) {
+    if (!h->two_streams || n_seg < 2 || first_stored == 0 || use_persist(h)) {
         for (int seg = n_seg - 1; seg >= 0; --seg) {
-            const bool resident = seg >= first_res;
-            const SegSet ss = resident ? res_set(h, seg - first_res) : seg_set(h, 0);
-            if (!resident && (rc = recompute_segment(h, seg, T, ss, st))) return rc;
+            const SegSet ss = set_of(seg);
+            if (seg < first_stored && (rc = recompute_segment(h, seg, T, ss, st))) return rc;
             if ((rc = adjoint_segment(h, seg, T, ss, adj, adj_next, st))) return rc;
             std::swap(adj, adj_next);
         }
         return MPM_OK;
     }
-    // recomputation one segment ahead on the second stream; the last
-    // recomputed segment starts at once, beside the resident segments' adjoint
+    // recomputation one segment ahead on the second stream.  Segment s goes
+    // into set s & 1, which is free at once (the last two segments, when the
+    // forward pass stored none) or when the adjoint of segment s + 2 is done.
     cudaStream_t aux = h->aux_stream;
     MPM_CUDA(h, cudaEventRecord(h->ev_fork, st));
     MPM_CUDA(h, cudaStreamWaitEvent(aux, h->ev_fork, 0));
-    const int last = first_res - 1;
-    if ((rc = recompute_segment(h, last, T, seg_set(h, last & 1), aux))) return rc;
-    MPM_CUDA(h, cudaEventRecord(h->ev_rec[last & 1], aux));
+    auto recompute = [&](int s) -> int {
+        if (s + 2 < first_res) MPM_CUDA(h, cudaStreamWaitEvent(aux, h->ev_adj[s & 1], 0));
+        if ((rc = recompute_segment(h, s, T, seg_set(h, s & 1), aux))) return rc;
+        MPM_CUDA(h, cudaEventRecord(h->ev_rec[s & 1], aux));
+        return MPM_OK;
+    };
+    int next = first_stored - 1;  // the next segment to recompute
+    // without a tail, the last recomputed segment starts beside the resident
+    // segments' adjoint
+    if (h->n_tail == 0 && (rc = recompute(next--))) return rc;
     for (int seg = n_seg - 1; seg >= 0; --seg) {
-        if (seg >= first_res) {
-            if ((rc = adjoint_segment(h, seg, T, res_set(h, seg - first_res), adj, adj_next, st))) return rc;
-            std::swap(adj, adj_next);
-            continue;
-        }
-        if (seg >= 1) {
-            // set (seg-1)&1 was last read by the adjoint of segment seg+1
-            if (seg + 1 <= last) MPM_CUDA(h, cudaStreamWaitEvent(aux, h->ev_adj[(seg + 1) & 1], 0));
-            if ((rc = recompute_segment(h, seg - 1, T, seg_set(h, (seg - 1) & 1), aux))) return rc;
-            MPM_CUDA(h, cudaEventRecord(h->ev_rec[(seg - 1) & 1], aux));
-        }
-        MPM_CUDA(h, cudaStreamWaitEvent(st, h->ev_rec[seg & 1], 0));
-        if ((rc = adjoint_segment(h, seg, T, seg_set(h, seg & 1), adj, adj_next, st))) return rc;
-        MPM_CUDA(h, cudaEventRecord(h->ev_adj[seg & 1], st));
+        if (seg < first_res && next >= 0 && next >= seg - 1 && (rc = recompute(next--))) return rc;
+        if (seg < first_stored) MPM_CUDA(h, cudaStreamWaitEvent(st, h->ev_rec[seg & 1], 0));
+        if ((rc = adjoint_segment(h, seg, T, set_of(seg), adj, adj_next, st))) return rc;
+        if (seg < first_res) MPM_CUDA(h, cudaEventRecord(h->ev_adj[seg & 1], st));
         std::swap(adj, adj_next);
     }
     return MPM_OK;
@@ -1268,13 +1301,16 @@ int backward_pass(mpm_handle* h, cudaStream_t st) {
 int run_pass(mpm_handle* h, int pass, cudaStream_t st) {
     auto body = [&](cudaStream_t s) { return pass == 0 ? forward_pass(h, s) : backward_pass(h, s); };
     if (!h->graphs) return body(st);
-    if (!h->exec[pass]) {
+    const int form = h->n_tail > 0 ? 1 : 0;
+    cudaGraphExec_t& exec = h->exec[pass][form];
+    if (!exec) {
         long long launches_before = h->launches;
         long long cls_before[kNumClasses];
         for (int c = 0; c < kNumClasses; ++c) cls_before[c] = h->cls_issued[c];
         MPM_CUDA(h, cudaStreamBeginCapture(h->cap_stream, cudaStreamCaptureModeThreadLocal));
         h->capturing = true;
         h->capture_pass = pass;
+        h->capture_form = form;
         int rc = body(h->cap_stream);
         h->capturing = false;
         cudaGraph_t graph = nullptr;
@@ -1284,23 +1320,24 @@ int run_pass(mpm_handle* h, int pass, cudaStream_t st) {
             return rc;
         }
         if (e != cudaSuccess) return fail(h, MPM_ERR_CUDA, std::string("graph capture: ") + cudaGetErrorString(e));
-        e = cudaGraphInstantiate(&h->exec[pass], graph, 0);
+        e = cudaGraphInstantiate(&exec, graph, 0);
         cudaGraphDestroy(graph);
         if (e != cudaSuccess) {
-            h->exec[pass] = nullptr;
+            exec = nullptr;
             return fail(h, MPM_ERR_CUDA, std::string("graph instantiate: ") + cudaGetErrorString(e));
         }
-        h->graph_launches[pass] = h->launches - launches_before;
+        h->graph_launches[pass][form] = h->launches - launches_before;
         h->launches = launches_before;
         for (int c = 0; c < kNumClasses; ++c) {
-            h->graph_cls[pass][c] = h->cls_issued[c] - cls_before[c];
+            h->graph_cls[pass][form][c] = h->cls_issued[c] - cls_before[c];
             h->cls_issued[c] = cls_before[c];
         }
     }
-    MPM_CUDA(h, cudaGraphLaunch(h->exec[pass], st));
-    h->launches += h->graph_launches[pass];
-    for (int c = 0; c < kNumClasses; ++c) h->cls_issued[c] += h->graph_cls[pass][c];
+    MPM_CUDA(h, cudaGraphLaunch(exec, st));
+    h->launches += h->graph_launches[pass][form];
+    for (int c = 0; c < kNumClasses; ++c) h->cls_issued[c] += h->graph_cls[pass][form][c];
     h->ran_graph[pass] = true;
+    h->ran_form[pass] = form;
     return MPM_OK;
 }
 
@@ -1315,6 +1352,20 @@ int finish(mpm_handle* h, int pass, cudaStream_t st) {
         if (rc == MPM_OK) rc = r2;
     }
     return rc;
+}
+
+// 3D lists: the recomputation sets as a recomputation, or a forward pass that
+// stores its tail in them, expects them (accumulators, flags, counts and boxes
+// zero) where a pass over every node, a failed pass or a tail that no
+// backward consumed left them set.
+int clean_segments(mpm_handle* h, cudaStream_t st) {
+    if (!h->blocks || !h->grid_blocks || !(h->seg_dirty || h->seg_filled)) return MPM_OK;
+    MPM_CUDA(h, cudaMemsetAsync(h->seg_acc, 0, sizeof(float4) * 2 * h->total_nodes * h->K, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->blk_flag + 2 * h->n_blocks, 0, sizeof(int) * 2 * h->n_blocks, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->blk_count + 2, 0, sizeof(int) * 2, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->blk_wbox + 2 * h->n_wbox, 0, sizeof(int4) * 2 * h->n_wbox, st));
+    h->seg_dirty = h->seg_filled = false;
+    return MPM_OK;
 }
 
 int forward_impl(mpm_handle* h, const float* x0, const float* v0, const float* phi,
@@ -1349,6 +1400,11 @@ int forward_impl(mpm_handle* h, const float* x0, const float* v0, const float* p
         MPM_CUDA(h, cudaMemsetAsync(h->res_wbox, 0, sizeof(int4) * r * h->n_wbox, st));
         h->res_dirty = false;
     }
+    h->n_tail = h->last_used ? tail_segments(h) : 0;
+    h->last_used = false;
+    h->stored_tail = 0;
+    if (h->n_tail > 0 && (rc = clean_segments(h, st))) return rc;
+    if (h->n_tail > 0 && h->blocks) (h->grid_blocks ? h->seg_filled : h->seg_dirty) = true;
     if ((rc = run_pass(h, 0, st))) return rc;
     if (h->n_res > 0 && h->blocks && !h->grid_blocks) h->res_dirty = true;
     if ((rc = dcopy(h, loss_out, h->st_loss, sizeof(float) * h->n_inst, st))) return rc;
@@ -1359,6 +1415,7 @@ int forward_impl(mpm_handle* h, const float* x0, const float* v0, const float* p
     rc = finish(h, 0, st);
     if (rc != MPM_OK) return rc;
     h->forward_done = true;
+    h->stored_tail = h->n_tail;
     return MPM_OK;
 }
 
@@ -1369,16 +1426,12 @@ int backward_impl(mpm_handle* h, const float* dloss, float* g_phi, float* g_mag,
     const int d = h->dim;
     int rc;
     if ((rc = dcopy(h, h->dloss, dloss, sizeof(float) * h->n_inst, st))) return rc;
-    if (h->blocks && h->grid_blocks && h->seg_dirty) {
-        // the last backward pass ran over every node and left the segment
-        // accumulators set; the lists expect them zero
-        MPM_CUDA(h, cudaMemsetAsync(h->seg_acc, 0, sizeof(float4) * 2 * h->total_nodes * h->K, st));
-        MPM_CUDA(h, cudaMemsetAsync(h->blk_flag + 2 * h->n_blocks, 0, sizeof(int) * 2 * h->n_blocks, st));
-        MPM_CUDA(h, cudaMemsetAsync(h->blk_count + 2, 0, sizeof(int) * 2, st));
-        MPM_CUDA(h, cudaMemsetAsync(h->blk_wbox + 2 * h->n_wbox, 0, sizeof(int4) * 2 * h->n_wbox, st));
-        h->seg_dirty = false;
-    }
+    h->last_used = true;
+    h->n_tail = h->stored_tail;
+    h->stored_tail = 0;  // the adjoint empties the sets, and older segments go through them
+    if (h->n_tail == 0 && (rc = clean_segments(h, st))) return rc;
     if ((rc = run_pass(h, 1, st))) return rc;
+    h->seg_filled = false;
     if (h->blocks && !h->grid_blocks) h->seg_dirty = h->res_dirty = true;
     if (g_phi && (rc = dcopy(h, g_phi, h->gphi_d, sizeof(float) * h->Nd, st))) return rc;
     if (g_mag && (rc = dcopy(h, g_mag, h->gmag_d, sizeof(float) * d * h->Nd, st))) return rc;
@@ -1478,6 +1531,8 @@ int autotune_impl(mpm_handle* h, const char* cache_path, int sample_substeps, cu
         return MPM_OK;
     }
     const int sample = sample_substeps > 0 ? sample_substeps : 2 * h->K;
+    h->n_tail = 0;
+    if (int rc0 = clean_segments(h, st)) return rc0;
     const bool saved_graphs = h->graphs;
     const int saved_timing = h->timing_stride;
     h->timing_stride = 0;
