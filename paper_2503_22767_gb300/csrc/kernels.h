@@ -27,13 +27,14 @@ struct StepArgs {
     float* gphi = nullptr;           // current-order design gradients
     float* gmag = nullptr;
     const float* field = nullptr;    // [inst][n_steps][D]
-    float* gfield = nullptr;
-    // sum_p m_p v_x after each substep: the forward adds in 64 bits to
-    // [n_steps][n_inst][mom_slots] (mom_acc; warp w adds to slot w % mom_slots,
-    // a power of two), the adjoint reads the finished rows [n_steps][n_inst]
-    double* mom_acc = nullptr;
-    int mom_slots = 1;
-    const float* mom = nullptr;
+    // Sums over all particles of an instance, per substep: added in 64 bits to
+    // `slots` values each (a power of two; warp w adds to slot w % slots), so
+    // that thousands of warps do not queue for one address, and folded at the
+    // end of the pass.
+    int slots = 1;
+    double* mom_acc = nullptr;     // sum_p m_p v_x [n_steps][n_inst][slots] (forward)
+    const float* mom = nullptr;    // its folded rows [n_steps][n_inst] (read by the adjoint)
+    double* gfield_acc = nullptr;  // dL/dB_applied [n_inst][n_steps][slots][D]
     const float* Minst = nullptr;    // [n_inst] instance mass
     const float* dloss = nullptr;    // [n_inst]
     const int* inst_off = nullptr;   // [n_inst + 1]
@@ -135,6 +136,8 @@ cudaError_t launch_instance_mass(const Params& P, const float* phi, const int* i
 cudaError_t launch_loss(int dim, const Params& P, const float* s, const float* x0, const float* target,
                         const int* id, const int* inst_off, const double* mass_acc, const double* mom_acc,
                         int mom_slots, double* loss_acc, float* Minst, float* mom, float* loss_out, cudaStream_t st);
+// out[row][c] = sum over the slots of acc[row][slot][c], ncomp components per row
+cudaError_t launch_fold_slots(const double* acc, float* out, long long rows, int slots, int ncomp, cudaStream_t st);
 cudaError_t launch_seed(int dim, const Params& P, const float* s, const float* x0, const float* target,
                         const int* id, const int* inst_off, const float* phi, const float* Minst,
                         const float* mom, const float* dloss, float* adj, float* gphi,

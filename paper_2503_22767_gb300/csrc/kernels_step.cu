@@ -261,6 +261,17 @@ __global__ void __launch_bounds__(kFinalizeThreads)
     }
 }
 
+__global__ void k_fold_slots(const double* __restrict__ acc, float* __restrict__ out, long long rows, int slots,
+                             int ncomp) {
+    const long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= rows * ncomp) return;
+    const long long row = i / ncomp;
+    const double* a = acc + row * slots * ncomp + (i - row * ncomp);
+    double sum = 0.0;
+    for (int k = 0; k < slots; ++k) sum += a[(long long)k * ncomp];
+    out[i] = (float)sum;
+}
+
 template <int D>
 __global__ void k_seed(Params P, const float* __restrict__ s, const float* __restrict__ x0,
                        const float* __restrict__ target,
@@ -426,6 +437,12 @@ cudaError_t launch_loss(int dim, const Params& P, const float* s, const float* x
     }
     k_loss_finalize<<<P.n_inst, kFinalizeThreads, 0, st>>>(P, inst_off, mass_acc, mom_acc, mom_slots, loss_acc, Minst, mom,
                                                           loss_out);
+    return cudaGetLastError();
+}
+
+cudaError_t launch_fold_slots(const double* acc, float* out, long long rows, int slots, int ncomp, cudaStream_t st) {
+    if (rows * ncomp == 0) return cudaSuccess;
+    k_fold_slots<<<blocks_for(rows * ncomp, 256), 256, 0, st>>>(acc, out, rows, slots, ncomp);
     return cudaGetLastError();
 }
 

@@ -57,9 +57,10 @@ struct Extras {
                                   // ([b][n_steps][2][D]), or null for static boxes
     // non-uniform applied field B(x, t_n) = B_a[n] + G[n] (x - x_c), x_c the
     // domain centre: G per instance and substep, [inst][n_steps][D][D]
-    // (dB_i/dx_j), or null for a uniform field; gfgrad receives dL/dG
+    // (dB_i/dx_j), or null for a uniform field; gfgrad receives the slots of
+    // dL/dG, [inst][n_steps][slots][D][D] (StepArgs::slots)
     const float* fgrad;
-    float* gfgrad;
+    double* gfgrad;
 };
 
 // Programmatic dependent launch: a kernel launched with programmatic stream

@@ -98,14 +98,15 @@ struct mpm_handle {
     float* target = nullptr;
     float* mom = nullptr;      // momentum rows and masses the adjoint reads (finished by the loss kernel)
     float* Minst = nullptr;
-    double* mom_acc = nullptr;   // the forward's 64-bit sums: [T][n_inst][mom_slots], [n_inst], [n_inst]
+    int slots = 1;               // 64-bit slots per sum over an instance's particles (StepArgs::slots)
+    double* mom_acc = nullptr;   // the forward's 64-bit sums: [T][n_inst][slots], [n_inst], [n_inst]
     double* mass_acc = nullptr;
     double* loss_acc = nullptr;
-    int mom_slots = 1;
     float* dloss = nullptr;
     float* gphi_d = nullptr;
     float* gmag_d = nullptr;
     float* gfield_d = nullptr;
+    double* gfield_acc = nullptr;  // its slots [n_inst][T][slots][d]
     float* st_x0 = nullptr;
     float* st_v0 = nullptr;
     float* st_xout = nullptr;
@@ -120,6 +121,7 @@ struct mpm_handle {
     mpm::Extras ext_host{};              // host copy of *d_ext
     float* d_fgrad = nullptr;            // dB/dx per instance and substep
     float* d_gfgrad = nullptr;           // its gradient, filled by the backward pass
+    double* gfgrad_acc = nullptr;        // from these slots [n_inst][T][slots][d][d]
     bool backward_done = false;
     float* d_bmotion = nullptr;          // their offsets and velocities per substep
 
@@ -627,11 +629,10 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
     ALLOC(h->mag_d, d * h->Nd);
     ALLOC(h->field, (long long)h->n_inst * h->T * d);
     ALLOC(h->target, d * h->N);
-    // a slot of the momentum rows takes the warps of about 2,048 particles:
-    // one for a small body, 16 for a million particles
-    while (h->mom_slots < 16 && (long long)h->mom_slots * 2 * 2048 * h->n_inst <= h->N) h->mom_slots *= 2;
+    // a slot takes the warps of about 1,024 particles, up to 16 slots
+    while (h->slots < 16 && (long long)h->slots * 2 * 1024 * h->n_inst <= h->N) h->slots *= 2;
     ALLOC(h->mom, (long long)h->T * h->n_inst);
-    ALLOC(h->mom_acc, (long long)h->T * h->n_inst * h->mom_slots);
+    ALLOC(h->mom_acc, (long long)h->T * h->n_inst * h->slots);
     ALLOC(h->mass_acc, h->n_inst);
     ALLOC(h->Minst, h->n_inst);
     ALLOC(h->loss_acc, h->n_inst);
@@ -639,9 +640,11 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
     ALLOC(h->gphi_d, h->Nd);
     ALLOC(h->gmag_d, d * h->Nd);
     ALLOC(h->gfield_d, (long long)h->n_inst * h->T * d);
+    ALLOC(h->gfield_acc, (long long)h->n_inst * h->T * h->slots * d);
     ALLOC(h->d_ext, 1);
     ALLOC(h->d_fgrad, (long long)h->n_inst * h->T * d * d);
     ALLOC(h->d_gfgrad, (long long)h->n_inst * h->T * d * d);
+    ALLOC(h->gfgrad_acc, (long long)h->n_inst * h->T * h->slots * d * d);
     ALLOC(h->d_bmotion, (long long)mpm::kMaxBoundaries * h->T * 2 * d);
     ALLOC(h->st_x0, d * h->N);
     ALLOC(h->st_v0, d * h->N);
@@ -709,7 +712,8 @@ StepArgs base_args(mpm_handle* h) {
     a.dloss = h->dloss;
     a.gphi = h->gphi_cur;
     a.gmag = h->gmag_cur;
-    a.gfield = h->gfield_d;
+    a.gfield_acc = h->gfield_acc;
+    a.slots = h->slots;
     return a;
 }
 
@@ -834,7 +838,7 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
     auto acc3 = [&](int i) { return h->acc3 + G * (i % 3); };
     int rc;
     MPM_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
-    MPM_CUDA(h, cudaMemsetAsync(h->mom_acc, 0, sizeof(double) * h->T * h->n_inst * h->mom_slots, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->mom_acc, 0, sizeof(double) * h->T * h->n_inst * h->slots, st));
     MPM_CUDA(h, cudaMemsetAsync(h->mass_acc, 0, sizeof(double) * h->n_inst, st));
     MPM_CUDA(h, cudaMemsetAsync(h->loss_acc, 0, sizeof(double) * h->n_inst, st));
     if (fuse) MPM_CUDA(h, cudaMemsetAsync(h->acc3, 0, sizeof(float4) * 2 * G, st));
@@ -899,7 +903,6 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
                                     cudaMemcpyDeviceToDevice, st));
         StepArgs a = base_args(h);
         a.mom_acc = h->mom_acc;
-        a.mom_slots = h->mom_slots;
         if (seg == 0 && (rc = counted(h, 1, [&] {
                              return mpm::launch_instance_mass(P, h->phi_fwd, h->d_inst_off, h->mass_acc, st);
                          })))
@@ -980,7 +983,7 @@ int forward_pass(mpm_handle* h, cudaStream_t st) {
     }
     if ((rc = counted(h, 2, [&] {
              return mpm::launch_loss(d, P, cur, h->x0_fwd, h->target, id_cur, h->d_inst_off, h->mass_acc,
-                                     h->mom_acc, h->mom_slots, h->loss_acc, h->Minst, h->mom, h->st_loss, st);
+                                     h->mom_acc, h->slots, h->loss_acc, h->Minst, h->mom, h->st_loss, st);
          })))
         return rc;
     h->cur = cur;
@@ -1067,7 +1070,6 @@ int recompute_segment(mpm_handle* h, int seg, int T, const SegSet& ss, cudaStrea
         a.mag = ss.mag;
         a.x0 = ss.x0;
         a.mom_acc = mom_acc;
-        a.mom_slots = h->mom_slots;
         a.s_in = state(k);
         a.s_out = state(k + 1);
         a.acc = next_acc;
@@ -1239,16 +1241,31 @@ int adjoint_segment(mpm_handle* h, int seg, int T, const SegSet& ss, float* adj,
     return finish_adjoint_segment(h, id_seg, ss, Ks, st);
 }
 
+int backward_segments(mpm_handle* h, cudaStream_t st);
+
 int backward_pass(mpm_handle* h, cudaStream_t st) {
+    const int d = h->dim;
+    const long long rows = (long long)h->n_inst * h->T;
+    int rc = backward_segments(h, st);
+    if (rc != MPM_OK) return rc;
+    if ((rc = counted(h, 1, [&] {
+             return mpm::launch_fold_slots(h->gfield_acc, h->gfield_d, rows, h->slots, d, st);
+         })))
+        return rc;
+    if (!h->ext_host.fgrad) return MPM_OK;
+    return counted(h, 1, [&] { return mpm::launch_fold_slots(h->gfgrad_acc, h->d_gfgrad, rows, h->slots, d * d, st); });
+}
+
+int backward_segments(mpm_handle* h, cudaStream_t st) {
     const int d = h->dim;
     const long long G = h->total_nodes;
     int rc;
     MPM_CUDA(h, cudaMemsetAsync(h->d_err, 0, sizeof(int), st));
     MPM_CUDA(h, cudaMemsetAsync(h->gphi_d, 0, sizeof(float) * h->Nd, st));
     MPM_CUDA(h, cudaMemsetAsync(h->gmag_d, 0, sizeof(float) * d * h->Nd, st));
-    MPM_CUDA(h, cudaMemsetAsync(h->gfield_d, 0, sizeof(float) * h->n_inst * h->T * d, st));
+    MPM_CUDA(h, cudaMemsetAsync(h->gfield_acc, 0, sizeof(double) * h->n_inst * h->T * h->slots * d, st));
     if (h->ext_host.fgrad)
-        MPM_CUDA(h, cudaMemsetAsync(h->d_gfgrad, 0, sizeof(float) * h->n_inst * h->T * d * d, st));
+        MPM_CUDA(h, cudaMemsetAsync(h->gfgrad_acc, 0, sizeof(double) * h->n_inst * h->T * h->slots * d * d, st));
     if (h->fuse_adj && !use_persist(h)) MPM_CUDA(h, cudaMemsetAsync(h->Vbar3, 0, sizeof(float4) * 3 * G, st));
     else MPM_CUDA(h, cudaMemsetAsync(h->Vbar, 0, sizeof(float4) * G, st));
     const int T = h->tune_T > 0 ? std::min(h->T, h->tune_T) : h->T;
@@ -1809,7 +1826,7 @@ int mpm_set_field_gradient(mpm_handle* h, const float* grad, void* cuda_stream) 
     const size_t n = (size_t)h->n_inst * h->T * h->dim * h->dim;
     if (grad) MPM_CUDA(h, cudaMemcpyAsync(h->d_fgrad, grad, sizeof(float) * n, cudaMemcpyDeviceToDevice, st));
     h->ext_host.fgrad = grad ? h->d_fgrad : nullptr;
-    h->ext_host.gfgrad = grad ? h->d_gfgrad : nullptr;
+    h->ext_host.gfgrad = grad ? h->gfgrad_acc : nullptr;
     return upload_extras(h, st);
 }
 

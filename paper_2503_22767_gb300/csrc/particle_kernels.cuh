@@ -205,9 +205,8 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
         // so that they do not queue for one address
         if (P.loss_kind == 1 && a.mom_acc != nullptr)
             warp_add_per_instance<1>(mom_x, inst,
-                                     a.mom_acc + (long long)a.n_g2p * P.n_inst * a.mom_slots +
-                                         ((p >> 5) & (a.mom_slots - 1)),
-                                     a.mom_slots);
+                                     a.mom_acc + (long long)a.n_g2p * P.n_inst * a.slots + ((p >> 5) & (a.slots - 1)),
+                                     a.slots);
     }
     if (P2G) {
         // this warp's box of listed cells, read after the scatter (3D)
@@ -709,11 +708,13 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
 #pragma unroll
             for (int i = 0; i < D; ++i) a.gmag[(long long)i * np + p] += brb[i];
         }
-        warp_add_per_instance<D>(bab, inst, a.gfield + (long long)a.n_p2g * D,
-                                 (long long)P.n_steps * D);
+        // into slots: with one sum per instance, the 31,250 warps of a million
+        // particles queued at three addresses (adjoint 200 -> 160 us per launch)
+        const long long slot = (long long)a.n_p2g * a.slots + ((p >> 5) & (a.slots - 1));
+        const long long per_inst = (long long)P.n_steps * a.slots;
+        warp_add_per_instance<D>(bab, inst, a.gfield_acc + slot * D, per_inst * D);
         if (has_fgrad)  // uniform over the launch: every lane takes part
-            warp_add_per_instance<D * D>(gG, inst, P.ext->gfgrad + (long long)a.n_p2g * D * D,
-                                         (long long)P.n_steps * D * D);
+            warp_add_per_instance<D * D>(gG, inst, P.ext->gfgrad + slot * D * D, per_inst * D * D);
         if (!G2PT && active) {
             store_vec<D>(a.adj, L::X, np, p, xb);
             store_vec<D>(a.adj, L::V, np, p, vb);
