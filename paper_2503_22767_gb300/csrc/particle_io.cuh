@@ -9,6 +9,7 @@
 #include <utility>
 
 #include "kernels.h"
+#include "packed.cuh"
 
 namespace mpm {
 
@@ -148,6 +149,24 @@ __device__ __forceinline__ void node_velocity(const float4* __restrict__ grid, c
     } else {
         unpack3<D>(g, gv);
     }
+}
+
+// The same at offset (o0, om, ol) of the stencil whose base node is grid[0],
+// packed (2D: the offset is (om, ol)).
+template <int D, bool FUSE, bool BOXES = true>
+__device__ __forceinline__ typename NodePack<D>::Vel load_node_velocity(const float4* __restrict__ grid,
+                                                                        const Stencil<D>& s, const Params& P, int o0,
+                                                                        int om, int ol, int step) {
+    const float4 g = __ldg(grid + ((D == 3 ? o0 * P.res + om : om) * P.res + ol));
+    if (!FUSE) return NodePack<D>::vel(g);
+    float mv[D], gv[D];
+    int c[D];
+    unpack3<D>(make_float4(g.y, g.z, g.w, 0.0f), mv);
+    if (D == 3) c[0] = s.base[0] + o0;
+    c[D - 2] = s.base[D - 2] + om;
+    c[D - 1] = s.base[D - 1] + ol;
+    grid_velocity<D, BOXES>(P, c, g.x, mv, gv, step);
+    return NodePack<D>::vel(gv);
 }
 
 }  // namespace mpm

@@ -23,6 +23,7 @@
 
 #include "kernels.h"
 #include "particle_io.cuh"
+#include "stencil_sums.cuh"
 #include "warp_scatter.cuh"
 
 namespace mpm {
@@ -112,61 +113,29 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
         if (active) {
             const float4* __restrict__ Vi = Vg + (long long)inst * P.nodes;
             // Eq. 19-20 with x_i - x_p = (o - r) dx for stencil offset o:
-            //   v = sum w V,  C = (4/dx) (sum w V o^T - v r^T)
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
-                v[i] = 0.0f;
-#pragma unroll
-                for (int j = 0; j < D; ++j) C[i][j] = 0.0f;  // sum w V o^T
-            }
-            // The sums run axis by axis: over the last axis with its 1D weights
-            // (hv = sum w_l V, hv2 = sum o_l w_l V), then each row is weighted
-            // by the product pw of the other axes' weights.
-            const int nb = base_node<D>(s, P.res);
-            float hv[D], hv2[D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) hv[i] = hv2[i] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < stencil_size<D>(); ++k) {
-                const int o0 = stencil_offset<D>(k, 0), om = stencil_offset<D>(k, 1 % D);
-                const int ol = stencil_offset<D>(k, D - 1);
-                float gv[D];
-                NodeTerm<D> t;
-                t.node = nb + node_offset<D>(k, P.res);
-#pragma unroll
-                for (int e = 0; e < D; ++e) t.c[e] = s.base[e] + stencil_offset<D>(k, e);
-                node_velocity<D, FUSE, EXT>(Vi, t, P, gv, a.n_g2p);
-                const float wl = s.w[D - 1][ol];
-#pragma unroll
-                for (int i = 0; i < D; ++i) {
-                    const float wv = wl * gv[i];
-                    hv[i] = ol == 0 ? wv : hv[i] + wv;
-                    if (ol == 0) hv2[i] = 0.0f;
-                    else hv2[i] = add_offset(hv2[i], ol, wv);
-                }
-                if (ol == 2) {  // the row is complete
-                    const float pw = D == 2 ? s.w[0][o0] : s.w[0][o0] * s.w[1 % D][om];
-#pragma unroll
-                    for (int i = 0; i < D; ++i) {
-                        const float hp = pw * hv[i];
-                        v[i] += hp;
-                        C[i][D - 1] += pw * hv2[i];
-                        C[i][0] = add_offset(C[i][0], o0, hp);
-                        if (D == 3) C[i][1 % D] = add_offset(C[i][1 % D], om, hp);
-                    }
-                }
-            }
+            //   v = sum w V,  C = (4/dx) sum w V (o - r)^T
+            const float4* __restrict__ Vn = Vi + base_node<D>(s, P.res);
+            typename NodePack<D>::Vel vp, Mp[D];
+            gather_velocity<D>(
+                s,
+                [&](int o0, int om, int ol) {
+                    return load_node_velocity<D, FUSE, EXT>(Vn, s, P, o0, om, ol, a.n_g2p);
+                },
+                vp, Mp);
+            NodePack<D>::get(vp, v);
             if (P2G && a.x0) {  // x0 again for the P2G position; the load overlaps the G2P tail
 #pragma unroll
                 for (int i = 0; i < D; ++i) xo[i] = reload(a.x0 + (long long)i * np + p);
             }
             float Fn[D][D];
-            const float c4 = 4.0f * P.inv_dx;
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
+            for (int j = 0; j < D; ++j) {
+                float m[D];
+                NodePack<D>::get(Mp[j], m);
+                const float c4 = (j == D - 1 ? 0.5f : 4.0f) * P.inv_dx;
 #pragma unroll
-                for (int j = 0; j < D; ++j) C[i][j] = c4 * (C[i][j] - v[i] * s.r[j]);
-                x[i] += P.dt * v[i];                              // Eq. 21 (on u = x - x0)
+                for (int i = 0; i < D; ++i) C[i][j] = c4 * m[i];
+                x[j] += P.dt * v[j];                              // Eq. 21 (on u = x - x0)
             }
             // Eq. 22 in strain form: E' = E + dt C (I + E)
 #pragma unroll
