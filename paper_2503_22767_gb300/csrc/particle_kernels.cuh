@@ -246,51 +246,30 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
                 for (int j = 0; j < 3; ++j) s.w[i][j] = 0.0f;
             }
         }
-        if constexpr (AGG) {
-            // node (o0, .., ol) receives w (mp, u + A o), w = (w0 w1) w2 as below
-            scatter_aggregated<D>(nb, inst, active, a.acc, P.nodes, P.res, sm, [&](int k) {
-                const int o0 = stencil_offset<D>(k, 0), om = stencil_offset<D>(k, 1 % D);
-                const int ol = stencil_offset<D>(k, D - 1);
-                const float pw = D == 2 ? s.w[0][o0] : s.w[0][o0] * s.w[1 % D][om];
-                const float w = pw * s.w[D - 1][ol];
-                float mv[D];
+        // node (o0, .., ol) receives w (mp, u + dx A o)  (Eq. 14 in the first component)
+        using NP = NodePack<D>;
+        const typename NP::Mass U = NP::mass(mp, u);
+        typename NP::Mass As[D];
 #pragma unroll
-                for (int i = 0; i < D; ++i) {
-                    float t = add_offset(u[i], o0, A[i][0]);
-                    if (D == 3) t = add_offset(t, om, A[i][1 % D]);
-                    mv[i] = w * add_offset(t, ol, A[i][D - 1]);
-                }
-                return pack4<D>(w * mp, mv);
-            });
+        for (int j = 0; j < D; ++j) {
+            float col[D];
+#pragma unroll
+            for (int i = 0; i < D; ++i) col[i] = A[i][j];
+            As[j] = NP::mass(0.0f, col);
+        }
+        if constexpr (AGG) {
+            scatter_aggregated<D>(nb, inst, active, a.acc, P.nodes, P.res, sm,
+                                  NodeValues<D, typename NP::Mass>{s, U, As, U, 0.0f});
             // the warp lists the node blocks its stencils reach beyond its box
             // (a.blk is uniform over the launch, so the whole warp takes part)
             if constexpr (D == 3) {
                 if (a.blk.flag != nullptr) mark_blocks(a.blk, p >> 5, active, inst, s.base, P.res, a.blk.wbox[p >> 5]);
             }
         } else if (active) {
-            float pw = 0.0f, Ug[D];  // per row: product of the other axes' weights, u + dx A o
+            float4* __restrict__ an = ai + nb;
+            NodeValues<D, typename NP::Mass> value{s, U, As, U, 0.0f};
 #pragma unroll
-            for (int i = 0; i < D; ++i) Ug[i] = 0.0f;
-#pragma unroll
-            for (int k = 0; k < stencil_size<D>(); ++k) {
-                const int ol = stencil_offset<D>(k, D - 1);
-                if (ol == 0)
-                    pw = D == 2 ? s.w[0][stencil_offset<D>(k, 0)]
-                                : s.w[0][stencil_offset<D>(k, 0)] * s.w[1 % D][stencil_offset<D>(k, 1 % D)];
-                const float w = pw * s.w[D - 1][ol];
-                if (ol == 0) {  // a new row: u + dx A o over all but the last axis
-#pragma unroll
-                    for (int i = 0; i < D; ++i) {
-                        float ug = add_offset(u[i], stencil_offset<D>(k, 0), A[i][0]);
-                        if (D == 3) ug = add_offset(ug, stencil_offset<D>(k, 1 % D), A[i][1 % D]);
-                        Ug[i] = ug;
-                    }
-                }
-                float mv[D];
-#pragma unroll
-                for (int i = 0; i < D; ++i) mv[i] = w * add_offset(Ug[i], ol, A[i][D - 1]);
-                atomicAdd(ai + nb + node_offset<D>(k, P.res), pack4<D>(w * mp, mv));  // Eq. 14 in .x
-            }
+            for (int k = 0; k < stencil_size<D>(); ++k) atomicAdd(an + node_offset<D>(k, P.res), value(k));
         }
     }
     if (flags) atomicOr(a.err, flags);
@@ -836,20 +815,13 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
         }
         if constexpr (AGG) {
             // node (o0, .., ol) receives w sv, sv = q + kappa dx Ct o, as above
-            scatter_aggregated<D>(nb, inst, active, a.Vbar, P.nodes, P.res, sm, [&](int k) {
-                const int o0 = stencil_offset<D>(k, 0), om = stencil_offset<D>(k, 1 % D);
-                const int ol = stencil_offset<D>(k, D - 1);
-                const float pw = D == 2 ? s.w[0][o0] : s.w[0][o0] * s.w[1 % D][om];
-                const float w = pw * s.w[D - 1][ol];
-                float sv[D];
+            using NP = NodePack<D>;
+            const typename NP::Vel Q = NP::vel(q);
+            typename NP::Vel Cs[D];
 #pragma unroll
-                for (int i = 0; i < D; ++i) {
-                    float t = add_offset(q[i], o0, dC[0][i]);
-                    if (D == 3) t = add_offset(t, om, dC[1 % D][i]);
-                    sv[i] = w * add_offset(t, ol, dC[D - 1][i]);
-                }
-                return make_float4(sv[0], sv[1 % D], D == 3 ? sv[2 % D] : 0.0f, 0.0f);
-            });
+            for (int c = 0; c < D; ++c) Cs[c] = NP::vel(dC[c]);
+            scatter_aggregated<D>(nb, inst, active, a.Vbar, P.nodes, P.res, sm,
+                                  NodeValues<D, typename NP::Vel>{s, Q, Cs, Q, 0.0f});
         }
     }
     if (flags) atomicOr(a.err, flags);
