@@ -121,6 +121,42 @@ __device__ __forceinline__ void store_mat(float* __restrict__ s, int base, long 
         for (int b = 0; b < D; ++b) s[(long long)(base + a * D + b) * np + p] = M[a][b];
 }
 
+// Particle values parked in the warp's scatter slab while no register should
+// hold them: component c of a lane at float c * 32 + lane.  park() copies from
+// global memory without passing through registers (cp.async); a lane reads
+// back only its own copies, after park_wait().
+__device__ __forceinline__ void park(float4* sm, int c, const float* src) {
+    float* dst = reinterpret_cast<float*>(sm) + c * 32 + (threadIdx.x & 31);
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void park_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
+// all but the last N committed groups have arrived
+template <int N>
+__device__ __forceinline__ void park_wait() {
+    asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
+}
+// (volatile, as reload(): the value is read where it is written, not kept)
+__device__ __forceinline__ float parked(const float4* sm, int c) {
+    const float* src = reinterpret_cast<const float*>(sm) + c * 32 + (threadIdx.x & 31);
+    float v;
+    asm volatile("ld.shared.f32 %0, [%1];" : "=f"(v) : "r"((unsigned)__cvta_generic_to_shared(src)));
+    return v;
+}
+
+template <int D>
+__device__ __forceinline__ void park_mat(float4* sm, int c, const float* __restrict__ s, int base, long long np, int p) {
+#pragma unroll
+    for (int k = 0; k < D * D; ++k) park(sm, c + k, s + (long long)(base + k) * np + p);
+}
+template <int D>
+__device__ __forceinline__ void parked_mat(const float4* sm, int c, float (&M)[D][D]) {
+#pragma unroll
+    for (int a = 0; a < D; ++a)
+#pragma unroll
+        for (int b = 0; b < D; ++b) M[a][b] = parked(sm, c + a * D + b);
+}
+
 constexpr int kStencil2 = 9, kStencil3 = 27;
 template <int D>
 constexpr int stencil_size() { return D == 2 ? kStencil2 : kStencil3; }

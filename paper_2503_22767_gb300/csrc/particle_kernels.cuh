@@ -313,6 +313,14 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
     // particles: 119.3 -> 117.4 us).  The 2D budgets spill nothing in the
     // plain order and lose with this one (2D batch: 108.3 -> 112.3 us).
     constexpr bool kLate = RELIEF && D == 3;
+    // The matrices of the fused 3D kernel wait in the scatter slab (idle until
+    // the scatter at the end; 4 x 9 floats a lane fill it): C, E and Fbar of
+    // state n and E of state m, copied there without registers while the
+    // kernel still waits for its predecessor (as loads where each is used, C
+    // read three times and E twice: 3D plate, 3 x 200,000 particles, design
+    // gradient 16,220 us; parked: 15,955).
+    constexpr bool kPark = kLate && P2GT && G2PT;
+    constexpr int kParkC = 0, kParkE = D * D, kParkFb = 2 * D * D, kParkEm = 3 * D * D;
     const bool active = p < P.n_total;
     const int inst = active ? find_instance(a.inst_off, P.n_inst, p) : -1;
     const long long np = P.np;
@@ -326,6 +334,14 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
         load_vec<D>(a.s_in, L::V, np, p, v_n);
         // C and E are read again after the P2G^T node loop under RELIEF:
         // plain loads, so that the second read finds them cached
+        if (kPark) {
+            park_mat<D>(sm, kParkC, a.s_in, L::C, np, p);
+            park_mat<D>(sm, kParkE, a.s_in, L::F, np, p);
+            park_commit();
+            park_mat<D>(sm, kParkFb, a.adj, L::F, np, p);
+            park_mat<D>(sm, kParkEm, a.s_aux, L::F, np, p);
+            park_commit();
+        } else
 #pragma unroll
         for (int i = 0; i < D; ++i)
 #pragma unroll
@@ -344,8 +360,10 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
         // request them now so that their loads after P2G^T find them in L2
 #pragma unroll
         for (int c = 0; c < D; ++c) prefetch_l2(a.s_aux + (long long)(L::X + c) * np + p);
+        if (!kPark) {
 #pragma unroll
-        for (int c = 0; c < D * D; ++c) prefetch_l2(a.s_aux + (long long)(L::F + c) * np + p);
+            for (int c = 0; c < D * D; ++c) prefetch_l2(a.s_aux + (long long)(L::F + c) * np + p);
+        }
     }
     if (P2GT && active) {  // the design and its gradients, read late in P2G^T
         prefetch_l2(a.gphi + p);
@@ -389,6 +407,11 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             if (Gn) field_at_particle<D>(Gn, x, Ba);
             Stencil<D> s;
             if (!make_stencil<D>(x, P, s)) flags |= kErrDomain;
+            if (kPark) {
+                park_wait<1>();
+                parked_mat<D>(sm, kParkE, F);
+                parked_mat<D>(sm, kParkC, Cn);
+            }
             StressParts<D> S;
             stress_parts<D>(F, phi, P, S);
             piola<D>(S, Br, Ba, Pk);
@@ -530,7 +553,12 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             // cheaper than the spills); with registers to spare they stay live.
             // kLate: E, the stress and Fbar are formed only where first used,
             // and P element by element.
-            if (RELIEF) reload_mat<D>(a.s_in, L::C, np, p, Cn);
+            if (kPark) {
+                park_wait<0>();
+                parked_mat<D>(sm, kParkC, Cn);
+            } else if (RELIEF) {
+                reload_mat<D>(a.s_in, L::C, np, p, Cn);
+            }
             if (RELIEF && !kLate) reload_mat<D>(a.s_in, L::F, np, p, F);
             if (!kLate) load_mat<D>(a.adj, L::F, np, p, Fb);
             if (RELIEF && !kLate) {
@@ -565,7 +593,8 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
 #pragma unroll
                     for (int j = 0; j < D; ++j) Cb[i][j] = mp * Ab[i][j];
             }
-            if (kLate) reload_mat<D>(a.s_in, L::F, np, p, F);
+            if (kPark) parked_mat<D>(sm, kParkE, F);
+            else if (kLate) reload_mat<D>(a.s_in, L::F, np, p, F);
 #pragma unroll
             for (int i = 0; i < D; ++i)
 #pragma unroll
@@ -581,7 +610,8 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                 }
             if (kLate) {
                 stress_parts<D>(F, phi, P, S);
-                load_mat<D>(a.adj, L::F, np, p, Fb);
+                if (kPark) parked_mat<D>(sm, kParkFb, Fb);
+                else load_mat<D>(a.adj, L::F, np, p, Fb);
                 // P_kj as piola() forms it, used by its three products at once
                 const float smu = S.s * (1.0f / kMu0);
 #pragma unroll
@@ -686,11 +716,14 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             }
             float x[D], F[D][D];
             load_position<D>(a.s_aux, a.x0, np, p, x);  // the position x0 + u
-            load_mat<D>(a.s_aux, L::F, np, p, F);
+            if (kPark) parked_mat<D>(sm, kParkEm, F);
+            else load_mat<D>(a.s_aux, L::F, np, p, F);
             if (!make_stencil<D>(x, P, s)) flags |= kErrDomain;
             // x' = x + dt v',  F' = (I + dt C') F  (Eq. 21-22)
             float vt[D], Ct[D][D], Fo[D][D];
-            if (kLate && P2GT) reload_mat<D>(a.s_in, L::C, np, p, Cn);  // C of state n, for (I + dt C')^T
+            // C of state n, for (I + dt C')^T
+            if (kPark) parked_mat<D>(sm, kParkC, Cn);
+            else if (kLate && P2GT) reload_mat<D>(a.s_in, L::C, np, p, Cn);
 #pragma unroll
             for (int i = 0; i < D; ++i) vt[i] = vb[i] + P.dt * xb[i];
 #pragma unroll
