@@ -172,23 +172,10 @@ __device__ __forceinline__ void clear_buffer(const StepArgs& a) {
         a.zero4[i] = make_float4(0.f, 0.f, 0.f, 0.f);
 }
 
-// Grid velocity at a stencil node: read V (separate grid kernel) or apply
-// the grid operation (Eq. 16-18) to the node's accumulator (fused).
-template <int D, bool FUSE, bool BOXES = true>
-__device__ __forceinline__ void node_velocity(const float4* __restrict__ grid, const NodeTerm<D>& t,
-                                              const Params& P, float (&gv)[D], int step) {
-    const float4 g = __ldg(grid + t.node);
-    if (FUSE) {
-        float mv[D];
-        unpack3<D>(make_float4(g.y, g.z, g.w, 0.0f), mv);
-        grid_velocity<D, BOXES>(P, t.c, g.x, mv, gv, step);
-    } else {
-        unpack3<D>(g, gv);
-    }
-}
-
-// The same at offset (o0, om, ol) of the stencil whose base node is grid[0],
-// packed (2D: the offset is (om, ol)).
+// Grid velocity at offset (o0, om, ol) of the stencil whose base node is
+// grid[0] (2D: the offset is (om, ol)), packed: read from V (separate grid
+// kernel), or the grid operation (Eq. 16-18) applied to the node's
+// accumulator (fused).
 template <int D, bool FUSE, bool BOXES = true>
 __device__ __forceinline__ typename NodePack<D>::Vel load_node_velocity(const float4* __restrict__ grid,
                                                                         const Stencil<D>& s, const Params& P, int o0,
@@ -203,6 +190,28 @@ __device__ __forceinline__ typename NodePack<D>::Vel load_node_velocity(const fl
     c[D - 1] = s.base[D - 1] + ol;
     grid_velocity<D, BOXES>(P, c, g.x, mv, gv, step);
     return NodePack<D>::vel(gv);
+}
+
+// The adjoint (mbar, mvbar) of that node: from the grid adjoint kernel, or
+// (FUSE) the reverse of the grid operation on the node's accumulator grid[.]
+// and velocity adjoint vbar[.].
+template <int D, bool FUSE, bool BOXES = true>
+__device__ __forceinline__ typename NodePack<D>::Mass load_node_adjoint(const float4* __restrict__ grid,
+                                                                        const float4* __restrict__ vbar,
+                                                                        const Stencil<D>& s, const Params& P, int o0,
+                                                                        int om, int ol, int step) {
+    const int node = (D == 3 ? o0 * P.res + om : om) * P.res + ol;
+    const float4 g = __ldg(grid + node);
+    if (!FUSE) return NodePack<D>::mass(g);
+    float mv[D], vb[D], mvb[D], mb;
+    int c[D];
+    unpack3<D>(make_float4(g.y, g.z, g.w, 0.0f), mv);
+    unpack3<D>(__ldg(vbar + node), vb);
+    if (D == 3) c[0] = s.base[0] + o0;
+    c[D - 2] = s.base[D - 2] + om;
+    c[D - 1] = s.base[D - 1] + ol;
+    grid_velocity_adjoint<D, BOXES>(P, c, g.x, mv, vb, mb, mvb, step);
+    return NodePack<D>::mass(mb, mvb);
 }
 
 }  // namespace mpm

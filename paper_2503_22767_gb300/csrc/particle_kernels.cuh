@@ -426,25 +426,19 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                     A[i][j] = mp * Cn[i][j] - sc * pft;
                 }
             // Node sums with x_i - x_p = (o - r) dx (o the stencil offset):
-            //   S0 = sum w mvb,  T = sum w mvb o^T,  mbs = sum w mb
-            // give vbar = mp S0, Abar = dx (T - S0 r^T) and
+            //   S0 = sum w mvb,  T = sum w mvb (o - r)^T,  mbs = sum w mb
+            // give vbar = mp S0, Abar = dx T and
             // mbar_p = mbs + S0 . v + C : Abar.  The node's contribution to
             // the particle's momentum is
-            //   inner = mb mp + mvb . (mp v + A dpos) = mb mp + mvb . (u + dx A o),
-            // u = mp v - dx A r, and xbar += sum (grad w) inner - A^T S0.
-            // Every stencil sum runs axis by axis: over the last axis with its
-            // 1D weights, then the partial sums are weighted by the other
-            // axes' weights, so no node forms a product of weights.
+            //   mb mp + mvb . (mp v + dx A (o - r)),
+            // whose weighted sum's derivative with respect to r is dx xbar
+            // (adjoint_sums).
             float u[D], dA[D][D];  // dA[c][i] = dx A_ic
 #pragma unroll
             for (int i = 0; i < D; ++i) {
-                float ar = 0.0f;
 #pragma unroll
-                for (int j = 0; j < D; ++j) {
-                    ar += A[i][j] * s.r[j];
-                    dA[j][i] = P.dx * A[i][j];
-                }
-                u[i] = mp * v[i] - P.dx * ar;
+                for (int j = 0; j < D; ++j) dA[j][i] = P.dx * A[i][j];
+                u[i] = mp * v[i];
             }
             if (Gn) {  // the body force is part of the particle's momentum term
                 float f[D];
@@ -452,100 +446,25 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
 #pragma unroll
                 for (int i = 0; i < D; ++i) u[i] += P.dt * f[i];
             }
-            const float4* __restrict__ gi = (FUSE ? a.accP : a.gadj) + (long long)inst * P.nodes;
-            const float4* __restrict__ vbi = FUSE ? a.VbarIn + (long long)inst * P.nodes : nullptr;
+            using NP = NodePack<D>;
             const int nb = base_node<D>(s, P.res);
-            float S0[D], T[D][D], mbs = 0.0f, xg[D];
-            // partial sums over the last axis (h*) and, in 3D, the middle axis (l*)
-            float Ug[D], hv[D], hv2[D], hm = 0.0f, ha = 0.0f, hb = 0.0f, la = 0.0f, lb = 0.0f, lc = 0.0f;
+            const float4* __restrict__ gi = (FUSE ? a.accP : a.gadj) + (long long)inst * P.nodes + nb;
+            const float4* __restrict__ vbi = FUSE ? a.VbarIn + (long long)inst * P.nodes + nb : nullptr;
+            float S0[D], mbs, xg[D];
+            typename NP::Mom Tp[D];
+            {
+                typename NP::Mass Sp;
+                typename NP::Mom Ap[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                S0[i] = xg[i] = Ug[i] = hv[i] = hv2[i] = 0.0f;
-#pragma unroll
-                for (int j = 0; j < D; ++j) T[i][j] = 0.0f;
+                for (int c = 0; c < D; ++c) Ap[c] = NP::mom(dA[c]);
+                adjoint_sums<D, true>(
+                    s,
+                    [&](int o0, int om, int ol) {
+                        return load_node_adjoint<D, FUSE, EXT>(gi, vbi, s, P, o0, om, ol, a.n_p2g);
+                    },
+                    NP::mass(mp, u), Ap, Sp, Tp, xg);
+                NP::get(Sp, mbs, S0);
             }
-            auto node_loop = [&]() {
-#pragma unroll
-                for (int k = 0; k < stencil_size<D>(); ++k) {
-                    const int o0 = stencil_offset<D>(k, 0), om = stencil_offset<D>(k, 1 % D);
-                    const int ol = stencil_offset<D>(k, D - 1);
-                    if (ol == 0) {  // a new row along the last axis
-#pragma unroll
-                        for (int i = 0; i < D; ++i) {
-                            float ug = add_offset(u[i], o0, dA[0][i]);
-                            if (D == 3) ug = add_offset(ug, om, dA[1 % D][i]);
-                            Ug[i] = ug;
-                            hv[i] = hv2[i] = 0.0f;
-                        }
-                        hm = ha = hb = 0.0f;
-                    }
-                    float4 g;
-                    float mvb[D];
-                    if (FUSE) {
-                        const int node = nb + node_offset<D>(k, P.res);
-                        g = __ldg(gi + node);
-                        // grid adjoint (reverse of Eq. 16-18) of this node, on the fly
-                        int c[D];
-#pragma unroll
-                        for (int e = 0; e < D; ++e) c[e] = s.base[e] + stencil_offset<D>(k, e);
-                        float mv[D], vbv[D], mbv;
-                        unpack3<D>(make_float4(g.y, g.z, g.w, 0.0f), mv);
-                        unpack3<D>(__ldg(vbi + node), vbv);
-                        grid_velocity_adjoint<D, EXT>(P, c, g.x, mv, vbv, mbv, mvb, a.n_p2g);
-                        g.x = mbv;
-                    } else {
-                        g = __ldg(gi + nb + node_offset<D>(k, P.res));
-                        unpack3<D>(make_float4(g.y, g.z, g.w, 0.0f), mvb);
-                    }
-                    const float wl = s.w[D - 1][ol], dwl = s.dw[D - 1][ol];
-                    float inner = g.x * mp;
-#pragma unroll
-                    for (int i = 0; i < D; ++i) {
-                        inner += mvb[i] * add_offset(Ug[i], ol, dA[D - 1][i]);
-                        const float wm = wl * mvb[i];
-                        hv[i] += wm;
-                        if (ol == 1) hv2[i] += wm;
-                        else if (ol == 2) hv2[i] += 2.0f * wm;
-                    }
-                    hm += wl * g.x;
-                    ha += wl * inner;
-                    hb += dwl * inner;
-                    if (ol == 2) {  // the row is complete: weight it by the other axes
-                        const float w0 = s.w[0][o0], dw0 = s.dw[0][o0];
-                        float pw = w0;
-                        if (D == 2) {
-                            xg[0] += dw0 * ha;
-                            xg[D - 1] += w0 * hb;
-                        } else {
-                            const float w1 = s.w[1 % D][om], dw1 = s.dw[1 % D][om];
-                            if (om == 0) la = lb = lc = 0.0f;
-                            la += w1 * ha;
-                            lb += dw1 * ha;
-                            lc += w1 * hb;
-                            if (om == 2) {
-                                xg[0] += dw0 * la;
-                                xg[1 % D] += w0 * lb;
-                                xg[D - 1] += w0 * lc;
-                            }
-                            pw = w0 * w1;
-                        }
-                        mbs += pw * hm;
-#pragma unroll
-                        for (int i = 0; i < D; ++i) {
-                            const float hp = pw * hv[i];
-                            S0[i] += hp;
-                            T[i][D - 1] += pw * hv2[i];
-                            if (o0 == 1) T[i][0] += hp;
-                            else if (o0 == 2) T[i][0] += 2.0f * hp;
-                            if (D == 3) {
-                                if (om == 1) T[i][1 % D] += hp;
-                                else if (om == 2) T[i][1 % D] += 2.0f * hp;
-                            }
-                        }
-                    }
-                }
-            };
-            node_loop();
             // The node loop needs none of C, E, the stress (all used for A
             // before it) and Fbar of state n.  Under a tight register budget
             // (RELIEF) they are read again, and the stress recomputed, here, so
@@ -565,23 +484,17 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                 stress_parts<D>(F, phi, P, S);
                 piola<D>(S, Br, Ba, Pk);
             }
-            // grad w is (dw along its own axis) / dx times the other weights;
-            // A^T S0 = (dA S0) / dx
-#pragma unroll
-            for (int c = 0; c < D; ++c) {
-                float g = xg[c];
-#pragma unroll
-                for (int i = 0; i < D; ++i) g -= dA[c][i] * S0[i];
-                xb[c] += P.inv_dx * g;
-            }
             float Ab[D][D], mpb = mbs;
 #pragma unroll
-            for (int i = 0; i < D; ++i) {
-                vb[i] = mp * S0[i];
-                mpb += S0[i] * v[i];
+            for (int j = 0; j < D; ++j) {
+                float tj[D];
+                NP::get_mom(Tp[j], tj);
+                xb[j] += P.inv_dx * xg[j];
+                vb[j] = mp * S0[j];
+                mpb += S0[j] * v[j];
 #pragma unroll
-                for (int j = 0; j < D; ++j) {
-                    Ab[i][j] = P.dx * (T[i][j] - S0[i] * s.r[j]);
+                for (int i = 0; i < D; ++i) {
+                    Ab[i][j] = (j == D - 1 ? 0.125f : 1.0f) * P.dx * tj[i];
                     mpb += Cn[i][j] * Ab[i][j];
                 }
             }
@@ -740,13 +653,11 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                     Fo[i][j] = ctf;
                 }
             store_mat<D>(a.adj, L::F, np, p, Fo);  // complete: the stencil sums add nothing to it
-            const float4* __restrict__ Vi = (FUSE_V ? a.accG : a.V) + (long long)inst * P.nodes;
+            using NP = NodePack<D>;
             // Eq. 19-20 reversed (v' = sum w V, C' = kappa sum w V dpos^T) with
             // dpos = (o - r) dx: the node's velocity adjoint is w sv,
             //   sv = vt + kappa Ct dpos = q + kappa dx Ct o,  q = vt - kappa dx Ct r,
-            // and xbar += sum (grad w) (V . sv) - kappa Ct^T sum w V.  The stencil
-            // sums run axis by axis as in P2G^T; only the scatter needs the
-            // node's weight.
+            // and dx xbar += d/dr sum w V . sv (adjoint_sums).
             const float kdx = P.kappa * P.dx;
 #pragma unroll
             for (int i = 0; i < D; ++i) {
@@ -759,81 +670,30 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                 q[i] = vt[i] - kdx * cr;
             }
             nb = base_node<D>(s, P.res);
-            float xg[D], vs[D], Sg[D], hv[D], pw = 0.0f, ha = 0.0f, hb = 0.0f, la = 0.0f, lb = 0.0f, lc = 0.0f;
+            const float4* __restrict__ Vn = (FUSE_V ? a.accG : a.V) + (long long)inst * P.nodes + nb;
+            float xg[D];
+            {
+                typename NP::Vel Cp[D], Vs, none[D];
 #pragma unroll
-            for (int i = 0; i < D; ++i) xg[i] = vs[i] = Sg[i] = hv[i] = 0.0f;
-            auto node_loop = [&]() {
-#pragma unroll
-                for (int k = 0; k < stencil_size<D>(); ++k) {
-                    const int o0 = stencil_offset<D>(k, 0), om = stencil_offset<D>(k, 1 % D);
-                    const int ol = stencil_offset<D>(k, D - 1);
-                    if (ol == 0) {  // a new row along the last axis
-#pragma unroll
-                        for (int i = 0; i < D; ++i) {
-                            float sg = add_offset(q[i], o0, dC[0][i]);
-                            if (D == 3) sg = add_offset(sg, om, dC[1 % D][i]);
-                            Sg[i] = sg;
-                            hv[i] = 0.0f;
-                        }
-                        ha = hb = 0.0f;
-                        pw = D == 2 ? s.w[0][o0] : s.w[0][o0] * s.w[1 % D][om];
-                    }
-                    const int node = nb + node_offset<D>(k, P.res);
-                    float gv[D];
-                    {
-                        NodeTerm<D> t;
-                        t.node = node;
-#pragma unroll
-                        for (int e = 0; e < D; ++e) t.c[e] = s.base[e] + stencil_offset<D>(k, e);
-                        node_velocity<D, FUSE_V, EXT>(Vi, t, P, gv, a.n_p2g - 1);
-                    }
-                    const float wl = s.w[D - 1][ol], dwl = s.dw[D - 1][ol];
-                    float sv[D], dot = 0.0f;
-#pragma unroll
-                    for (int i = 0; i < D; ++i) {
-                        sv[i] = add_offset(Sg[i], ol, dC[D - 1][i]);
-                        dot += gv[i] * sv[i];  // V . (vt + kappa Ct dpos)
-                        hv[i] += wl * gv[i];
-                    }
-                    ha += wl * dot;
-                    hb += dwl * dot;
-                    if constexpr (!AGG) {
-                        const float w = pw * wl;
-#pragma unroll
-                        for (int i = 0; i < D; ++i) sv[i] *= w;
-                        atomicAdd(Vbi + node, make_float4(sv[0], sv[1 % D], D == 3 ? sv[2 % D] : 0.0f, 0.0f));
-                    }
-                    if (ol == 2) {  // the row is complete: weight it by the other axes
-                        const float w0 = s.w[0][o0], dw0 = s.dw[0][o0];
-                        if (D == 2) {
-                            xg[0] += dw0 * ha;
-                            xg[D - 1] += w0 * hb;
-                        } else {
-                            const float w1 = s.w[1 % D][om], dw1 = s.dw[1 % D][om];
-                            if (om == 0) la = lb = lc = 0.0f;
-                            la += w1 * ha;
-                            lb += dw1 * ha;
-                            lc += w1 * hb;
-                            if (om == 2) {
-                                xg[0] += dw0 * la;
-                                xg[1 % D] += w0 * lb;
-                                xg[D - 1] += w0 * lc;
-                            }
-                        }
-#pragma unroll
-                        for (int i = 0; i < D; ++i) vs[i] += pw * hv[i];
-                    }
-                }
-            };
-            node_loop();
-            // kappa Ct^T vs = (dC vs) / dx
-#pragma unroll
-            for (int c = 0; c < D; ++c) {
-                float g = xg[c];
-#pragma unroll
-                for (int i = 0; i < D; ++i) g -= dC[c][i] * vs[i];
-                xb[c] += P.inv_dx * g;
+                for (int c = 0; c < D; ++c) Cp[c] = NP::vel(dC[c]);
+                adjoint_sums<D, false>(
+                    s,
+                    [&](int o0, int om, int ol) {
+                        return load_node_velocity<D, FUSE_V, EXT>(Vn, s, P, o0, om, ol, a.n_p2g - 1);
+                    },
+                    NP::vel(vt), Cp, Vs, none, xg);
             }
+            if constexpr (!AGG) {
+                typename NP::Vel Cp[D];
+#pragma unroll
+                for (int c = 0; c < D; ++c) Cp[c] = NP::vel(dC[c]);
+                const typename NP::Vel Q = NP::vel(q);
+                NodeValues<D, typename NP::Vel> value{s, Q, Cp, Q, 0.0f};
+#pragma unroll
+                for (int k = 0; k < stencil_size<D>(); ++k) atomicAdd(Vbi + nb + node_offset<D>(k, P.res), value(k));
+            }
+#pragma unroll
+            for (int c = 0; c < D; ++c) xb[c] += P.inv_dx * xg[c];
             store_vec<D>(a.adj, L::X, np, p, xb);
         } else {  // a lane past the end takes part in the aggregated scatter with zeros
 #pragma unroll
