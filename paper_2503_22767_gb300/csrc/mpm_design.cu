@@ -90,90 +90,111 @@ __global__ void k_filter_order_cells(const int* __restrict__ counts, const int* 
     }
 }
 
-// out_p = sum_{|x_p' - x_p| < R} (1 - |x_p' - x_p| / R) val_p'  (Eq. 23-24),
-// divided by norm_p when norm is given; val == nullptr sums the weights
-// alone (the normaliser W_p).  One thread per particle, in cell order.
-template <int D>
-__global__ void __launch_bounds__(256) k_filter_apply(const float* __restrict__ x0, int n, FilterGrid g,
-                                                      const int* __restrict__ order,
-                                                      const int* __restrict__ offsets,
-                                                      const float* __restrict__ val,
-                                                      const float* __restrict__ norm, float* __restrict__ out) {
-    int t = blockIdx.x * blockDim.x + threadIdx.x;
-    if (t >= n) return;
-    const int p = order[t];
-    float x[D];
-    int c[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) x[a] = x0[(long long)a * n + p];
-    cell_of<D>(x, g, c);
-    int lo[D], hi[D];
-#pragma unroll
-    for (int a = 0; a < D; ++a) {
-        lo[a] = max(c[a] - 1, 0);
-        hi[a] = min(c[a] + 1, g.nc - 1);
-    }
-    const float rR = 1.0f / g.R;
-    float acc = 0.0f;
-    int cc[D];
-    // visit the (up to) 3^d neighbour cells
-    for (int k = 0; k < (D == 2 ? 9 : 27); ++k) {
-        int r = k;
-        bool in = true;
-#pragma unroll
-        for (int a = D - 1; a >= 0; --a) {
-            cc[a] = c[a] - 1 + r % 3;
-            r /= 3;
-            in = in && cc[a] >= lo[a] && cc[a] <= hi[a];
-        }
-        if (!in) continue;
-        const int cell = cell_index<D>(cc, g.nc);
-        const int j1 = offsets[cell + 1];
-        for (int j = offsets[cell]; j < j1; ++j) {
-            const int q = order[j];
-            float d2 = 0.0f;
-#pragma unroll
-            for (int a = 0; a < D; ++a) {
-                const float dx = x0[(long long)a * n + q] - x[a];
-                d2 += dx * dx;
-            }
-            const float dist = sqrtf(d2);
-            if (dist < g.R) {
-                const float w = 1.0f - dist * rR;
-                acc += val ? w * val[q] : w;
-            }
-        }
-    }
-    out[p] = norm ? acc / norm[p] : acc;
-}
-
-// Eq. 25 and its reverse
+// Eq. 25
 __device__ __forceinline__ float heaviside(float x, float beta, float t_half) {
     return (t_half + tanhf(beta * (x - 0.5f))) / (2.0f * t_half);
 }
 
-__global__ void k_heaviside(const float* __restrict__ phi_t, int n, float beta, float t_half,
-                            float* __restrict__ phi_bar) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p < n) phi_bar[p] = heaviside(phi_t[p], beta, t_half);
+template <int D>
+__global__ void k_filter_positions(const float* __restrict__ x0, int n, const int* __restrict__ order,
+                                   float4* __restrict__ sorted) {
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const int p = order[t];
+    // value 1: the sum over the neighbours is then the normaliser W_p
+    sorted[t] = make_float4(x0[p], x0[(long long)n + p], D == 3 ? x0[2LL * n + p] : 0.0f, 1.0f);
 }
 
-// u_p = (dL/dphi_bar_p) dH/dphi~ / W_p: the vector the transposed filter gathers
-__global__ void k_heaviside_adjoint(const float* __restrict__ phi_t, const float* __restrict__ g, int n,
-                                    float beta, float t_half, const float* __restrict__ norm,
-                                    float* __restrict__ u) {
-    int p = blockIdx.x * blockDim.x + threadIdx.x;
-    if (p >= n) return;
-    const float th = tanhf(beta * (phi_t[p] - 0.5f));
-    u[p] = g[p] * beta * (1.0f - th * th) / (2.0f * t_half) / norm[p];
+// The filter's next input in cell order: val, or (REVERSE) the vector the
+// transposed filter gathers, u_p = (dL/dphi_bar_p) dH/dphi~ / W_p.
+template <bool REVERSE>
+__global__ void k_filter_values(const int* __restrict__ order, int n, const float* __restrict__ val,
+                                const float* __restrict__ phi_t, const float* __restrict__ norm, float beta,
+                                float t_half, float4* __restrict__ sorted) {
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const int p = order[t];
+    float v = val[p];
+    if (REVERSE) {
+        const float th = tanhf(beta * (phi_t[p] - 0.5f));
+        v = v * beta * (1.0f - th * th) / (2.0f * t_half) / norm[p];
+    }
+    sorted[t].w = v;
+}
+
+// out_p = sum_{|x_p' - x_p| < R} (1 - |x_p' - x_p| / R) val_p'  (Eq. 23-24),
+// divided by norm_p when norm is given; phi_bar_p = H(out_p) (Eq. 25) when
+// phi_bar is given.  One thread per particle, in cell order.  sorted holds
+// (position, val) of every particle in cell order, so the three neighbour
+// cells along the last axis are one contiguous range, read with one load per
+// candidate that the lanes of a cell share.  Most candidates (27 of 32 at
+// R = 1.5 cells) lie outside R: the square root is taken inside only (the
+// slack keeps its rounding from deciding differently than the exact test).
+// Bound by issue: 729 candidates per particle.  200,000 particles, R = 1.5
+// grid cells, the design maps with their reverse and the Adam steps: 560 us
+// with three ranges of indices into unsorted positions (four loads and a
+// square root per candidate), 308 us so.
+template <int D>
+__global__ void __launch_bounds__(256) k_filter_apply(const float4* __restrict__ sorted, int n, FilterGrid g,
+                                                      const int* __restrict__ order,
+                                                      const int* __restrict__ offsets,
+                                                      const float* __restrict__ norm, float beta, float t_half,
+                                                      float* __restrict__ out, float* __restrict__ phi_bar) {
+    int t = blockIdx.x * blockDim.x + threadIdx.x;
+    if (t >= n) return;
+    const float4 me = sorted[t];
+    float x[D];
+    int c[D];
+    x[0] = me.x, x[1] = me.y;
+    if (D == 3) x[2 % D] = me.z;
+    cell_of<D>(x, g, c);
+    const int l0 = max(c[D - 1] - 1, 0), l1 = min(c[D - 1] + 1, g.nc - 1);
+    const float rR = 1.0f / g.R, near2 = g.R * g.R * 1.00001f;
+    float acc = 0.0f;
+    auto add = [&](const float4& q) {
+        const float dx = q.x - me.x, dy = q.y - me.y;
+        float d2 = dx * dx + dy * dy;
+        if (D == 3) {
+            const float dz = q.z - me.z;
+            d2 += dz * dz;
+        }
+        if (d2 < near2) {
+            const float dist = sqrtf(d2);
+            if (dist < g.R) acc += (1.0f - dist * rR) * q.w;
+        }
+    };
+    const int a0 = D == 3 ? max(c[0] - 1, 0) : 0, a1 = D == 3 ? min(c[0] + 1, g.nc - 1) : 0;
+    for (int ca = a0; ca <= a1; ++ca)
+        for (int cb = max(c[D - 2] - 1, 0); cb <= min(c[D - 2] + 1, g.nc - 1); ++cb) {
+            const int row = (ca * g.nc + cb) * g.nc;
+            const int j1 = offsets[row + l1 + 1];
+            int j = offsets[row + l0];
+            for (; j + 4 <= j1; j += 4) {
+                const float4 q0 = sorted[j], q1 = sorted[j + 1], q2 = sorted[j + 2], q3 = sorted[j + 3];
+                add(q0);
+                add(q1);
+                add(q2);
+                add(q3);
+            }
+            for (; j < j1; ++j) add(sorted[j]);
+        }
+    const int p = order[t];
+    const float r = norm ? acc / norm[p] : acc;
+    out[p] = r;
+    if (phi_bar) phi_bar[p] = heaviside(r, beta, t_half);
 }
 
 // Eq. 26-28
 template <int D>
 __global__ void k_magnetization(const float* __restrict__ Br, const float* __restrict__ zeta,
                                 const int* __restrict__ region, int n, int n_m, float Br_max, float delta,
-                                float* __restrict__ mag) {
+                                float* __restrict__ mag, float* __restrict__ keep_Br, float* __restrict__ keep_zeta) {
     int p = blockIdx.x * blockDim.x + threadIdx.x;
+    if (p < n_m) {  // the inputs, for the reverse
+        keep_Br[p] = Br[p];
+#pragma unroll
+        for (int i = 0; i < D; ++i) keep_zeta[(long long)i * n_m + p] = zeta[(long long)i * n_m + p];
+    }
     if (p >= n) return;
     const int r = region ? region[p] : p;
     float z[D], s2 = delta;
@@ -243,10 +264,17 @@ __global__ void __launch_bounds__(256) k_magnetization_adjoint(
 template <int D>
 __global__ void k_stimulus(const float* __restrict__ Ba, const float* __restrict__ f, const float* __restrict__ eta,
                            int n_tasks, int n_steps, float dt, float B_max, float f_min, float f_max, float delta,
-                           float* __restrict__ field) {
+                           float* __restrict__ field, float* __restrict__ keep_Ba, float* __restrict__ keep_f,
+                           float* __restrict__ keep_eta) {
     long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= (long long)n_tasks * n_steps) return;
     const int l = (int)(i / n_steps), s = (int)(i % n_steps);
+    if (s == 0) {  // the inputs, for the reverse
+        keep_Ba[l] = Ba[l];
+        keep_f[l] = f[l];
+#pragma unroll
+        for (int c = 0; c < D; ++c) keep_eta[l * D + c] = eta[l * D + c];
+    }
     float e[D], s2 = delta;
 #pragma unroll
     for (int c = 0; c < D; ++c) {
@@ -356,13 +384,12 @@ struct mpm_design {
     int n_m = 0;
     FilterGrid grid{};
     long long n_cells = 0;
-    float* x0 = nullptr;       // [d][N]
+    float4* sorted = nullptr;  // x_p(0) and the filter's current input, in cell order
     int* region = nullptr;     // [N] or null
     int* order = nullptr;      // particles in cell order
     int* offsets = nullptr;    // [n_cells + 1]
     float* norm = nullptr;     // W_p
     float* phi_t = nullptr;    // phi~ of the last forward
-    float* u = nullptr;        // reverse scratch
     float* in_Br = nullptr;    // material and stimulus inputs of the last forward:
     float* in_zeta = nullptr;  //   Br [n_m], zeta [d][n_m], Ba, f [n_tasks],
     float* in_Ba = nullptr;    //   eta [n_tasks][d]
@@ -387,10 +414,22 @@ int fail(mpm_design* h, int code, const std::string& why) {
     } while (0)
 
 void release(mpm_design* h) {
-    for (void* ptr : {(void*)h->x0, (void*)h->region, (void*)h->order, (void*)h->offsets, (void*)h->norm,
-                      (void*)h->phi_t, (void*)h->u, (void*)h->in_Br, (void*)h->in_zeta, (void*)h->in_Ba,
+    for (void* ptr : {(void*)h->sorted, (void*)h->region, (void*)h->order, (void*)h->offsets, (void*)h->norm,
+                      (void*)h->phi_t, (void*)h->in_Br, (void*)h->in_zeta, (void*)h->in_Ba,
                       (void*)h->in_f, (void*)h->in_eta})
         if (ptr) cudaFree(ptr);
+}
+
+cudaError_t filter_apply(const mpm_design* h, const float* norm, float beta, float t_half, float* out, float* phi_bar,
+                         cudaStream_t st) {
+    const int n = h->cfg.n_particles;
+    if (h->cfg.dim == 2)
+        k_filter_apply<2><<<blocks(n), 256, 0, st>>>(h->sorted, n, h->grid, h->order, h->offsets, norm, beta, t_half, out,
+                                                     phi_bar);
+    else
+        k_filter_apply<3><<<blocks(n), 256, 0, st>>>(h->sorted, n, h->grid, h->order, h->offsets, norm, beta, t_half, out,
+                                                     phi_bar);
+    return cudaGetLastError();
 }
 
 int create_impl(mpm_design* h, const mpm_design_config* c, const float* x0, const int* region, cudaStream_t st) {
@@ -411,10 +450,10 @@ int create_impl(mpm_design* h, const mpm_design_config* c, const float* x0, cons
     const long long tmp_len = mpm::sort_scan_tmp_len(h->n_cells + 1);
     int *keys = nullptr, *slot = nullptr, *counts = nullptr, *tmp = nullptr, *bad = nullptr;
     auto alloc = [&](void** p, size_t bytes) { return cudaMalloc(p, bytes > 0 ? bytes : 4) == cudaSuccess; };
-    bool ok = alloc((void**)&h->x0, sizeof(float) * d * (size_t)n) && alloc((void**)&h->order, sizeof(int) * (size_t)n) &&
+    bool ok = alloc((void**)&h->sorted, sizeof(float4) * (size_t)n) && alloc((void**)&h->order, sizeof(int) * (size_t)n) &&
               alloc((void**)&h->offsets, sizeof(int) * (size_t)(h->n_cells + 1)) &&
               alloc((void**)&h->norm, sizeof(float) * (size_t)n) && alloc((void**)&h->phi_t, sizeof(float) * (size_t)n) &&
-              alloc((void**)&h->u, sizeof(float) * (size_t)n) && alloc((void**)&keys, sizeof(int) * (size_t)n) &&
+              alloc((void**)&keys, sizeof(int) * (size_t)n) &&
               alloc((void**)&slot, sizeof(int) * (size_t)n) &&
               alloc((void**)&counts, sizeof(int) * (size_t)(h->n_cells + 1)) &&
               alloc((void**)&tmp, sizeof(int) * (size_t)tmp_len) && alloc((void**)&bad, sizeof(int)) &&
@@ -433,7 +472,6 @@ int create_impl(mpm_design* h, const mpm_design_config* c, const float* x0, cons
         if (rc == MPM_OK && e != cudaSuccess) rc = fail(h, MPM_ERR_CUDA, std::string(what) + ": " + cudaGetErrorString(e));
     };
     if (rc == MPM_OK) {
-        step(cudaMemcpyAsync(h->x0, x0, sizeof(float) * d * (size_t)n, cudaMemcpyDeviceToDevice, st), "copy x0");
         if (region) {
             step(cudaMemcpyAsync(h->region, region, sizeof(int) * (size_t)n, cudaMemcpyDeviceToDevice, st), "copy region");
             step(cudaMemsetAsync(bad, 0, sizeof(int), st), "memset");
@@ -442,8 +480,8 @@ int create_impl(mpm_design* h, const mpm_design_config* c, const float* x0, cons
         }
         step(cudaMemsetAsync(counts, 0, sizeof(int) * (size_t)(h->n_cells + 1), st), "memset");
         if (n > 0) {
-            if (d == 2) k_filter_keys<2><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, keys, slot, counts);
-            else k_filter_keys<3><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, keys, slot, counts);
+            if (d == 2) k_filter_keys<2><<<blocks(n), 256, 0, st>>>(x0, n, h->grid, keys, slot, counts);
+            else k_filter_keys<3><<<blocks(n), 256, 0, st>>>(x0, n, h->grid, keys, slot, counts);
             step(cudaGetLastError(), "k_filter_keys");
         }
         // offsets over n_cells + 1 entries: the last one is the total
@@ -453,14 +491,11 @@ int create_impl(mpm_design* h, const mpm_design_config* c, const float* x0, cons
             step(cudaGetLastError(), "k_filter_scatter");
             k_filter_order_cells<<<blocks(h->n_cells), 256, 0, st>>>(counts, h->offsets, h->order, h->n_cells);
             step(cudaGetLastError(), "k_filter_order_cells");
+            if (d == 2) k_filter_positions<2><<<blocks(n), 256, 0, st>>>(x0, n, h->order, h->sorted);
+            else k_filter_positions<3><<<blocks(n), 256, 0, st>>>(x0, n, h->order, h->sorted);
+            step(cudaGetLastError(), "k_filter_positions");
             // normalisers W_p = sum_p' w_pp'
-            if (d == 2)
-                k_filter_apply<2><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, nullptr,
-                                                             nullptr, h->norm);
-            else
-                k_filter_apply<3><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, nullptr,
-                                                             nullptr, h->norm);
-            step(cudaGetLastError(), "k_filter_apply");
+            step(filter_apply(h, nullptr, 0.0f, 0.0f, h->norm, nullptr, st), "k_filter_apply");
         }
     }
     int bad_h = 0;
@@ -531,34 +566,27 @@ int mpm_design_forward(mpm_design* h, float beta, const float* phi, const float*
     h->forward_done = false;
     const float t_half = tanhf(0.5f * beta);
     if (n > 0) {
+        k_filter_values<false><<<blocks(n), 256, 0, st>>>(h->order, n, phi, nullptr, nullptr, 0.0f, 0.0f, h->sorted);
+        DCUDA(h, cudaGetLastError());
+        DCUDA(h, filter_apply(h, h->norm, beta, t_half, h->phi_t, phi_bar, st));
+        const unsigned nb = blocks(n > h->n_m ? n : h->n_m);
         if (d == 2)
-            k_filter_apply<2><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, phi, h->norm, h->phi_t);
+            k_magnetization<2><<<nb, 256, 0, st>>>(Br, zeta, h->region, n, h->n_m, (float)c.Br_max, (float)c.delta, mag,
+                                                   h->in_Br, h->in_zeta);
         else
-            k_filter_apply<3><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, phi, h->norm, h->phi_t);
-        DCUDA(h, cudaGetLastError());
-        k_heaviside<<<blocks(n), 256, 0, st>>>(h->phi_t, n, beta, t_half, phi_bar);
-        DCUDA(h, cudaGetLastError());
-        if (d == 2) k_magnetization<2><<<blocks(n), 256, 0, st>>>(Br, zeta, h->region, n, h->n_m, (float)c.Br_max, (float)c.delta, mag);
-        else k_magnetization<3><<<blocks(n), 256, 0, st>>>(Br, zeta, h->region, n, h->n_m, (float)c.Br_max, (float)c.delta, mag);
+            k_magnetization<3><<<nb, 256, 0, st>>>(Br, zeta, h->region, n, h->n_m, (float)c.Br_max, (float)c.delta, mag,
+                                                   h->in_Br, h->in_zeta);
         DCUDA(h, cudaGetLastError());
     }
     const long long nf = (long long)c.n_tasks * c.n_steps;
-    auto keep = [&](float* dst, const float* src, long long count) {
-        return count > 0 ? cudaMemcpyAsync(dst, src, sizeof(float) * count, cudaMemcpyDeviceToDevice, st) : cudaSuccess;
-    };
-    if (n > 0) {
-        DCUDA(h, keep(h->in_Br, Br, h->n_m));
-        DCUDA(h, keep(h->in_zeta, zeta, (long long)d * h->n_m));
-    }
-    DCUDA(h, keep(h->in_Ba, Ba, c.n_tasks));
-    DCUDA(h, keep(h->in_f, f, c.n_tasks));
-    DCUDA(h, keep(h->in_eta, eta, (long long)d * c.n_tasks));
     if (d == 2)
         k_stimulus<2><<<blocks(nf), 256, 0, st>>>(Ba, f, eta, c.n_tasks, c.n_steps, (float)c.dt, (float)c.B_max,
-                                                  (float)c.f_min, (float)c.f_max, (float)c.delta, field);
+                                                  (float)c.f_min, (float)c.f_max, (float)c.delta, field, h->in_Ba,
+                                                  h->in_f, h->in_eta);
     else
         k_stimulus<3><<<blocks(nf), 256, 0, st>>>(Ba, f, eta, c.n_tasks, c.n_steps, (float)c.dt, (float)c.B_max,
-                                                  (float)c.f_min, (float)c.f_max, (float)c.delta, field);
+                                                  (float)c.f_min, (float)c.f_max, (float)c.delta, field, h->in_Ba,
+                                                  h->in_f, h->in_eta);
     DCUDA(h, cudaGetLastError());
     h->beta = beta;
     h->forward_done = true;
@@ -577,13 +605,10 @@ int mpm_design_backward(mpm_design* h, const float* g_phi_bar, const float* g_ma
     const float t_half = tanhf(0.5f * h->beta);
     if (n > 0) {
         // topology: Eq. 25 reversed, then the transposed filter of Eq. 23
-        k_heaviside_adjoint<<<blocks(n), 256, 0, st>>>(h->phi_t, g_phi_bar, n, h->beta, t_half, h->norm, h->u);
+        k_filter_values<true><<<blocks(n), 256, 0, st>>>(h->order, n, g_phi_bar, h->phi_t, h->norm, h->beta, t_half,
+                                                         h->sorted);
         DCUDA(h, cudaGetLastError());
-        if (d == 2)
-            k_filter_apply<2><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, h->u, nullptr, g_phi);
-        else
-            k_filter_apply<3><<<blocks(n), 256, 0, st>>>(h->x0, n, h->grid, h->order, h->offsets, h->u, nullptr, g_phi);
-        DCUDA(h, cudaGetLastError());
+        DCUDA(h, filter_apply(h, nullptr, 0.0f, 0.0f, g_phi, nullptr, st));
         // material: Eq. 26-28 reversed, summed per region
         const bool regions = h->region != nullptr;
         const bool stage = regions && (1 + d) * n_m <= kSmemRegionFloats;
