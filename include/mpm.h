@@ -85,7 +85,10 @@ typedef enum {
  *                     checkpoints, keeping every substep of the segment it
  *                     works on; 0 = one segment over the whole horizon.  With
  *                     MPM_OPT_RESIDENT_SEGMENTS the forward pass keeps the
- *                     last segments instead.
+ *                     last segments instead.  A forward pass whose predecessor
+ *                     was followed by a backward (a design loop) keeps its last
+ *                     two (before the resident ones) in the recomputation
+ *                     buffers, and the next backward starts with those.
  */
 typedef struct {
     int dim;

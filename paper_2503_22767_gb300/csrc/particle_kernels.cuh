@@ -35,10 +35,10 @@ namespace mpm {
 // (<= 128 registers), 3 (<= 80) and, in 2D, 4 (<= 64) blocks, chosen per
 // launch (Params::adj_blocks; 4 acts as 3 in 3D).
 constexpr int kMinBlocksForward3 = 4;
-// 2D: at most 48 registers (40 warps per SM, no spills); the 2D batch's
-// forward launch went from 83 to 79 us, the single 2D locomotion body is
-// unchanged (its 469 blocks of 64 threads are far from filling the GPU)
-constexpr int kMinBlocksForward2 = 5;
+// 2D: with the aggregated P2G (large launches) at most 48 registers (40 warps
+// per SM, no spills; the 2D batch's forward launch went from 83 to 79 us);
+// with per-lane atomics 64 (a small body's blocks are far from filling the GPU)
+constexpr int kMinBlocksForward2 = 4, kMinBlocksForward2Agg = 5;
 
 namespace {
 
@@ -76,6 +76,22 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
     // the G2P node loop for P2G, so that it holds no registers in the loop
     float x[D], v[D], C[D][D], F[D][D], xo[D];
     float phi = 0.0f, mp = 0.0f;
+    // In 2D with per-lane atomics (small bodies: a chain of short launches)
+    // the design and field of P2G are loaded with the state, so that their
+    // latency passes while the kernel waits for its predecessor (half-size
+    // walker, forward only: 1,664 -> 1,607 us per 400 substeps, with 64
+    // instead of 48 registers allowed).  The launches that fill the GPU need
+    // the registers more: loaded early, the 2D batch lost 1.7%; in 3D, copied
+    // early into the scatter slab, 1,000,000 particles lost 8%.
+    constexpr bool kHoist = D == 2 && P2G && !AGG_P2G;
+    float Br[D], Ba[D];
+    auto load_design = [&]() {
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            Br[i] = a.mag[(long long)i * np + p];
+            Ba[i] = __ldg(a.field + ((long long)inst * P.n_steps + a.n_p2g) * D + i);
+        }
+    };
     auto position = [&](float (&pos)[D]) {
 #pragma unroll
         for (int i = 0; i < D; ++i) pos[i] = __fadd_rn(x[i], xo[i]);
@@ -91,6 +107,7 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
             load_vec<D>(a.s_in, L::V, np, p, v);
             load_mat<D>(a.s_in, L::C, np, p, C);
         }
+        if (kHoist) load_design();
     };
     if (kEarly && active) load_state();
     if (CHAIN) {
@@ -123,7 +140,7 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
                 },
                 vp, Mp);
             NodePack<D>::get(vp, v);
-            if (P2G && a.x0) {  // x0 again for the P2G position; the load overlaps the G2P tail
+            if (P2G && a.x0 && !kHoist) {  // x0 again for the P2G position; the load overlaps the G2P tail
 #pragma unroll
                 for (int i = 0; i < D; ++i) xo[i] = reload(a.x0 + (long long)i * np + p);
             }
@@ -191,12 +208,8 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
             StressParts<D> S;
             stress_parts<D>(F, phi, P, S);
             if (!(S.J > 0.0f)) flags |= kErrNumeric;
-            float Br[D], Ba[D], Pk[D][D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
-                Br[i] = a.mag[(long long)i * np + p];
-                Ba[i] = __ldg(a.field + ((long long)inst * P.n_steps + a.n_p2g) * D + i);
-            }
+            float Pk[D][D];
+            if (!kHoist) load_design();
             if (EXT && P.ext->fgrad) {
                 const float* Gn = P.ext->fgrad + ((long long)inst * P.n_steps + a.n_p2g) * D * D;
                 field_at_particle<D>(Gn, pos, Ba);
@@ -277,7 +290,7 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
 
 // 3D: at most 64 registers (32 warps per SM) to keep more gathers in flight
 template <int D, bool G2P, bool P2G, bool WRITE_ALL, bool FUSE, bool EXT, bool AGG = aggregate_scatter<D>()>
-__global__ void __launch_bounds__(256, D == 3 ? kMinBlocksForward3 : kMinBlocksForward2)
+__global__ void __launch_bounds__(256, D == 3 ? kMinBlocksForward3 : AGG ? kMinBlocksForward2Agg : kMinBlocksForward2)
     k_forward(Params P, StepArgs a) {
     extern __shared__ float4 s_warp[];
     forward_particle<D, G2P, P2G, WRITE_ALL, FUSE, EXT, true, AGG>(
@@ -329,7 +342,37 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
     float xb[D], vb[D], Cb[D][D], Fb[D][D];
     float Cn[D][D];  // C of state n (= m+1), needed by G2P^T
     float x_n[D], v_n[D], F_n[D][D], phi_n = 0.0f;  // state n and design (P2G^T)
+    // 2D: the design and field with the state, as in the forward kernel (2D
+    // walker's design gradient 5,355 -> 5,270 us; the 3D plate lost 0.5%)
+    float Br[D], Ba[D];
+    auto load_design = [&]() {
+#pragma unroll
+        for (int i = 0; i < D; ++i) {
+            Br[i] = a.mag[(long long)i * np + p];
+            Ba[i] = __ldg(a.field + ((long long)inst * P.n_steps + a.n_p2g) * D + i);
+        }
+    };
+    // 2D with registers to spare (the 128-register budget of small bodies): the
+    // adjoint of F, the state of m and the locomotion seed too (walker 5,160 ->
+    // 5,030 -> 4,860 us; the 64-register launches of the batch lost 1%)
+    constexpr bool kAhead = D == 2 && P2GT && G2PT && !RELIEF;
+    float x_m[D], F_m[D][D];
+    constexpr bool kSeed = D == 2 && !RELIEF;
+    float M_n = 0.0f, dl_n = 0.0f, mom_n = 0.0f;
+    auto load_seed = [&]() {
+        if (P.loss_kind == 1 && a.n_p2g >= 1) {
+            M_n = a.Minst[inst];
+            dl_n = a.dloss[inst];
+            mom_n = a.mom[(long long)(a.n_p2g - 1) * P.n_inst + inst];
+        }
+    };
     auto load_state_n = [&]() {
+        if (kSeed) load_seed();
+        if (kAhead) {
+            load_mat<D>(a.adj, L::F, np, p, Fb);
+            load_position<D>(a.s_aux, a.x0, np, p, x_m);
+            load_mat<D>(a.s_aux, L::F, np, p, F_m);
+        }
         load_position<D>(a.s_in, a.x0, np, p, x_n);  // the position x0 + u
         load_vec<D>(a.s_in, L::V, np, p, v_n);
         // C and E are read again after the P2G^T node loop under RELIEF:
@@ -353,6 +396,7 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             }
         load_vec<D>(a.adj, L::X, np, p, xb);
         phi_n = a.phi[p];
+        if (D == 2) load_design();
     };
     if (kEarly && active) load_state_n();
     if (P2GT && G2PT && active) {
@@ -398,12 +442,8 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             float(&F)[D][D] = F_n;
             const float phi = phi_n;
             const float mp = phi * P.rho0 * P.p_vol;
-            float Br[D], Ba[D], Pk[D][D], A[D][D];
-#pragma unroll
-            for (int i = 0; i < D; ++i) {
-                Br[i] = a.mag[(long long)i * np + p];
-                Ba[i] = __ldg(a.field + ((long long)inst * P.n_steps + n) * D + i);
-            }
+            float Pk[D][D], A[D][D];
+            if (D == 3) load_design();
             if (Gn) field_at_particle<D>(Gn, x, Ba);
             Stencil<D> s;
             if (!make_stencil<D>(x, P, s)) flags |= kErrDomain;
@@ -479,7 +519,7 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                 reload_mat<D>(a.s_in, L::C, np, p, Cn);
             }
             if (RELIEF && !kLate) reload_mat<D>(a.s_in, L::F, np, p, F);
-            if (!kLate) load_mat<D>(a.adj, L::F, np, p, Fb);
+            if (!kLate && !kAhead) load_mat<D>(a.adj, L::F, np, p, Fb);
             if (RELIEF && !kLate) {
                 stress_parts<D>(F, phi, P, S);
                 piola<D>(S, Br, Ba, Pk);
@@ -586,11 +626,11 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
             }
             // locomotion seed on state n (n >= 1), Eq. 40
             if (P.loss_kind == 1 && n >= 1) {
-                const float M = a.Minst[inst];
+                if (!kSeed) load_seed();
+                const float M = M_n, dl = dl_n;
                 if (M > 0.0f) {
-                    const float dl = a.dloss[inst];
                     const float rM = 1.0f / M;
-                    const float vbar = a.mom[(long long)(n - 1) * P.n_inst + inst] * rM;
+                    const float vbar = mom_n * rM;
                     vb[0] -= P.dt * mp * rM * dl;
                     gph -= P.dt * (v[0] - vbar) * rM * dl * P.rho0 * P.p_vol;
                 }
@@ -631,9 +671,18 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
                 load_mat<D>(a.s_in, L::C, np, p, Cn);
             }
             float x[D], F[D][D];
-            load_position<D>(a.s_aux, a.x0, np, p, x);  // the position x0 + u
-            if (kPark) parked_mat<D>(sm, kParkEm, F);
-            else load_mat<D>(a.s_aux, L::F, np, p, F);
+            if (kAhead) {
+#pragma unroll
+                for (int i = 0; i < D; ++i) {
+                    x[i] = x_m[i];
+#pragma unroll
+                    for (int j = 0; j < D; ++j) F[i][j] = F_m[i][j];
+                }
+            } else {
+                load_position<D>(a.s_aux, a.x0, np, p, x);  // the position x0 + u
+                if (kPark) parked_mat<D>(sm, kParkEm, F);
+                else load_mat<D>(a.s_aux, L::F, np, p, F);
+            }
             if (!make_stencil<D>(x, P, s)) flags |= kErrDomain;
             // x' = x + dt v',  F' = (I + dt C') F  (Eq. 21-22)
             float vt[D], Ct[D][D], Fo[D][D];
