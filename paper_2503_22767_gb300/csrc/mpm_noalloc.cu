@@ -17,9 +17,17 @@
 // context id, and its first call looks the address up again. Make the first
 // call on a device before any CUDA stream capture begins.
 //
-// Each call reads the device error flags back and synchronises its stream,
-// so a call on a stream that is capturing is refused before it enqueues any
-// work (MPM_ERR_ARG), which leaves the caller's capture intact.
+// Each call synchronises its stream and reads the error flags, so a call on a
+// stream that is capturing is refused before it enqueues any work
+// (MPM_ERR_ARG), which leaves the caller's capture intact.
+//
+// A small body's call is a chain of latencies, so it is kept short: three
+// dependent launches (programmatic, so each is scheduled while its
+// predecessor drains), the accumulator left zero by the grid operation for
+// the next call instead of cleared by a launch of its own, and the error
+// flags in mapped host memory, which the kernels touch only on an error,
+// instead of a copy back.  2D beam of 1,024 particles through the Python
+// binding: 48.5 us per call before, 32 us so.
 //
 // The substep itself reuses the library's kernels: P2G (particle_kernels.cuh,
 // Eq. 14-15 with the stress of Eq. 7 / 31-33), the grid operation
@@ -40,14 +48,16 @@ constexpr long long kMaxNodes = MPM_NOALLOC_MAX_NODES;
 
 // [0, kMaxNodes): P2G accumulator (m, m v); [kMaxNodes, 2 kMaxNodes): grid velocity.
 static __device__ __align__(256) float4 g_noalloc_grid[2 * kMaxNodes];
-// [0], [1]: particle offsets of the single instance; [32]: device error flags.
-static __device__ __align__(256) int g_noalloc_misc[64];
 
 constexpr int kMaxDevices = 64;
 struct Scratch {
     unsigned long long ctx_id = 0;  // context the addresses belong to (0: none yet)
     float4* grid = nullptr;
-    int* misc = nullptr;
+    // error flags: one mapped page-locked word per device, as kernels see it
+    // (allocated in that context, and gone with it)
+    int* err_host = nullptr;
+    int* err = nullptr;
+    bool dirty = false;  // a call did not finish: the accumulator may not be zero
 };
 Scratch g_scratch[kMaxDevices];
 std::mutex g_scratch_mutex;
@@ -87,7 +97,8 @@ int current_context_id(unsigned long long* id, std::string* why) {
     return MPM_OK;
 }
 
-int scratch_for_current_device(Scratch* out, std::string* why) {
+// The scratch of the current device, marked dirty until finish_call(dev).
+int begin_call(Scratch* out, int* device, std::string* why) {
     int dev = -1;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) {
@@ -111,34 +122,32 @@ int scratch_for_current_device(Scratch* out, std::string* why) {
     Scratch& s = g_scratch[dev];
     if (s.ctx_id != ctx_id) {
         void* grid = nullptr;
-        void* misc = nullptr;
+        void* host = nullptr;
+        void* mapped = nullptr;
         e = cudaGetSymbolAddress(&grid, g_noalloc_grid);
-        if (e == cudaSuccess) e = cudaGetSymbolAddress(&misc, g_noalloc_misc);
+        if (e == cudaSuccess) e = cudaHostAlloc(&host, sizeof(int), cudaHostAllocMapped);
+        if (e == cudaSuccess && (e = cudaHostGetDevicePointer(&mapped, host, 0)) != cudaSuccess) cudaFreeHost(host);
         if (e != cudaSuccess) {
             cudaGetLastError();
-            *why = std::string("cudaGetSymbolAddress (loads the module and its 8 MiB scratch): ") +
-                   cudaGetErrorString(e);
+            *why = std::string("loading the module and its 8 MiB scratch: ") + cudaGetErrorString(e);
             return e == cudaErrorMemoryAllocation ? MPM_ERR_OOM : MPM_ERR_CUDA;
         }
         s.grid = static_cast<float4*>(grid);
-        s.misc = static_cast<int*>(misc);
+        s.err_host = static_cast<int*>(host);
+        s.err = static_cast<int*>(mapped);
+        s.dirty = false;  // the array starts zero with its module
         s.ctx_id = ctx_id;
     }
     *out = s;
+    *device = dev;
+    s.dirty = true;
     return MPM_OK;
 }
 
-// Clears the accumulator and the error flags left by the previous call and
-// writes the instance offsets {0, n}.
-__global__ void k_noalloc_setup(float4* __restrict__ acc, long long nodes, int* __restrict__ misc,
-                                int n) {
-    long long i = (long long)blockIdx.x * blockDim.x + threadIdx.x;
-    for (; i < nodes; i += (long long)gridDim.x * blockDim.x) acc[i] = make_float4(0.f, 0.f, 0.f, 0.f);
-    if (blockIdx.x == 0 && threadIdx.x == 0) {
-        misc[0] = 0;
-        misc[1] = n;
-        misc[32] = 0;
-    }
+// The calling thread's call on device dev has run to its end.
+void finish_call(int dev) {
+    std::lock_guard<std::mutex> lock(g_scratch_mutex);
+    g_scratch[dev].dirty = false;
 }
 
 int report(int code, const std::string& why) {
@@ -180,7 +189,8 @@ extern "C" int mpm_substep_noalloc(const mpm_config* cfg, int substep, const flo
                                    "back the device status and cannot be captured");
 
     Scratch sc;
-    rc = scratch_for_current_device(&sc, &why);
+    int dev = -1;
+    rc = begin_call(&sc, &dev, &why);
     if (rc != MPM_OK) return report(rc, why);
 
     const int d = cfg->dim;
@@ -190,6 +200,7 @@ extern "C" int mpm_substep_noalloc(const mpm_config* cfg, int substep, const flo
     P.wall_mode = cfg->wall_mode;
     P.loss_kind = cfg->loss_kind;
     P.simp_q = cfg->simp_q;
+    P.pdl = 1;
     P.n_inst = 1;
     P.n_steps = cfg->n_steps;
     P.n_total = n;
@@ -210,23 +221,22 @@ extern "C" int mpm_substep_noalloc(const mpm_config* cfg, int substep, const flo
 
     float4* acc = sc.grid;
     float4* V = sc.grid + kMaxNodes;
-    int* inst_off = sc.misc;
-    int* err = sc.misc + 32;
-    k_noalloc_setup<<<(unsigned)((nodes + 255) / 256), 256, 0, st>>>(acc, nodes, sc.misc, n);
-    if ((e = cudaGetLastError()) != cudaSuccess) return report(MPM_ERR_CUDA, cudaGetErrorString(e));
+    if (sc.dirty && (e = cudaMemsetAsync(acc, 0, sizeof(float4) * (size_t)kMaxNodes, st)) != cudaSuccess)
+        return report(MPM_ERR_CUDA, cudaGetErrorString(e));
+    volatile int* flags_host = sc.err_host;
+    *flags_host = 0;
 
     mpm::StepArgs a;
     a.s_in = state_in;
     a.phi = phi_bar;
     a.mag = mag;
     a.field = field;
-    a.inst_off = inst_off;
-    a.err = err;
+    a.err = sc.err;  // (one instance: the kernels look no particle offsets up)
     a.acc = acc;
     a.n_p2g = substep;
     if ((e = mpm::launch_forward(d, false, true, false, false, P, a, 128, st)) != cudaSuccess)
         return report(MPM_ERR_CUDA, cudaGetErrorString(e));
-    if ((e = mpm::launch_grid(d, P, acc, V, nullptr, false, substep, st)) != cudaSuccess)
+    if ((e = mpm::launch_grid(d, P, acc, V, nullptr, true, substep, st)) != cudaSuccess)
         return report(MPM_ERR_CUDA, cudaGetErrorString(e));
     mpm::StepArgs g = a;
     g.acc = nullptr;
@@ -236,10 +246,9 @@ extern "C" int mpm_substep_noalloc(const mpm_config* cfg, int substep, const flo
     if ((e = mpm::launch_forward(d, true, false, true, false, P, g, 128, st)) != cudaSuccess)
         return report(MPM_ERR_CUDA, cudaGetErrorString(e));
 
-    int flags = 0;
-    if ((e = cudaMemcpyAsync(&flags, err, sizeof(int), cudaMemcpyDeviceToHost, st)) != cudaSuccess ||
-        (e = cudaStreamSynchronize(st)) != cudaSuccess)
-        return report(MPM_ERR_CUDA, cudaGetErrorString(e));
+    if ((e = cudaStreamSynchronize(st)) != cudaSuccess) return report(MPM_ERR_CUDA, cudaGetErrorString(e));
+    finish_call(dev);
+    const int flags = *flags_host;
     if (flags & mpm::kErrDomain) return report(MPM_ERR_DOMAIN, "a particle stencil left the grid");
     if (flags & mpm::kErrNumeric) return report(MPM_ERR_NUMERIC, "inverted or non-finite deformation gradient");
     return MPM_OK;
