@@ -229,9 +229,10 @@ enum {
                            drains; 0: plain stream order */
     MPM_OPT_ADJOINT_BLOCKS = 8, /* register budget of the fused adjoint particle kernel, as
                            resident 256-thread blocks per SM: 2 (default in 2D, <= 128
-                           registers), 3 (default in 3D, <= 80 registers: more warps to hide
-                           gather latency, at the cost of spills) or 4 (<= 64 registers; 2D
-                           only, 3D takes it as 3) */
+                           registers), 3 (default in 3D, <= 80 registers, 96 in blocks of up
+                           to 128 threads: more warps to hide gather latency, at the cost of
+                           spills; a 3D body that one wave of 128-register warps holds takes
+                           those) or 4 (<= 64 registers; 2D only, 3D takes it as 3) */
     MPM_OPT_GRID_BLOCKS = 10, /* 3D: 1 (default): the P2G kernels list the blocks of 4x4x4
                            nodes their stencils touch, and the grid operation and its
                            reverse run over the listed blocks only; 0: over every node.

@@ -34,6 +34,7 @@ struct Params {
     int pdl;  // per-substep kernels launched with programmatic dependent launch
     int adj_blocks;  // register budget of the adjoint particle kernel: 256-thread blocks per SM (2 or 3)
     int agg2;        // 2D: the fused forward kernel's P2G scatter is aggregated over same-node lanes
+    int wave;        // 3D: particles that one wave of 128-register particle kernels holds (16 warps per SM)
     // solid boxes of Eq. 18 beyond the walls and a non-uniform applied field
     // (device memory), or null for neither.  One pointer keeps the parameter
     // block (and the transfer kernels' register allocation) as small as

@@ -668,6 +668,7 @@ int create_impl(const mpm_config* c, mpm_handle* h) {
         MPM_CUDA(h, cudaGetDevice(&dev));
         MPM_CUDA(h, cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev));
         h->grid_ctas = 4 * std::max(1, sms);
+        P.wave = 16 * 32 * std::max(1, sms);
         h->n_wbox = h->np / 32;
         ALLOC(h->blk_flag, 4 * h->n_blocks);
         ALLOC(h->blk_list, 4 * h->n_blocks);

@@ -34,7 +34,19 @@ namespace mpm {
 // kernel is held to 64 registers, and the adjoint kernel is compiled for 2
 // (<= 128 registers), 3 (<= 80) and, in 2D, 4 (<= 64) blocks, chosen per
 // launch (Params::adj_blocks; 4 acts as 3 in 3D).
+//
+// In 3D two rules go beyond the option.  A body that one wave of 128-register
+// kernels holds (Params::wave, 77,824 particles on 152 SMs) gains nothing from
+// more warps per SM, so both kernels take 128 registers: design gradient of
+// 64,000 particles 3,418 -> 3,069 us, of 14,304 1,493 -> 1,416; of 79,816, just
+// past the wave, it would lose 14%.  Larger bodies in blocks of up to 128
+// threads run the adjoint with five blocks of 128 threads per SM (96
+// registers, 36 instead of 244 bytes of spill loads): 64,000 particles 3,460
+// -> 3,380 us, 3 x 200,000 15,380 -> 15,335, 1,000,000 25.01 -> 24.91 ms;
+// blocks of 256 keep 80 registers (96 would leave two of them: +7%).
 constexpr int kMinBlocksForward3 = 4;
+constexpr int kMinBlocksOneWave = 2;
+constexpr int kBlocksOf128 = 5;  // MINB of the adjoint kernel for blocks of up to 128 threads
 // 2D: with the aggregated P2G (large launches) at most 48 registers (40 warps
 // per SM, no spills; the 2D batch's forward launch went from 83 to 79 us);
 // with per-lane atomics 64 (a small body's blocks are far from filling the GPU)
@@ -289,9 +301,13 @@ __device__ __forceinline__ void forward_particle(const Params& P, const StepArgs
 }
 
 // 3D: at most 64 registers (32 warps per SM) to keep more gathers in flight
-template <int D, bool G2P, bool P2G, bool WRITE_ALL, bool FUSE, bool EXT, bool AGG = aggregate_scatter<D>()>
-__global__ void __launch_bounds__(256, D == 3 ? kMinBlocksForward3 : AGG ? kMinBlocksForward2Agg : kMinBlocksForward2)
-    k_forward(Params P, StepArgs a) {
+template <int D, bool AGG>
+constexpr int forward_min_blocks() {
+    return D == 3 ? kMinBlocksForward3 : AGG ? kMinBlocksForward2Agg : kMinBlocksForward2;
+}
+template <int D, bool G2P, bool P2G, bool WRITE_ALL, bool FUSE, bool EXT, bool AGG = aggregate_scatter<D>(),
+          int MINB = forward_min_blocks<D, AGG>()>
+__global__ void __launch_bounds__(256, MINB) k_forward(Params P, StepArgs a) {
     extern __shared__ float4 s_warp[];
     forward_particle<D, G2P, P2G, WRITE_ALL, FUSE, EXT, true, AGG>(
         P, a, blockIdx.x * blockDim.x + threadIdx.x, s_warp + (threadIdx.x >> 5) * warp_slots<D, P2G, AGG>());
@@ -773,7 +789,7 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
 }
 
 template <int D, bool P2GT, bool G2PT, bool FUSE, bool FUSE_V, int MINB, bool EXT>
-__global__ void __launch_bounds__(256, MINB) k_adjoint(Params P, StepArgs a) {
+__global__ void __launch_bounds__(MINB == kBlocksOf128 ? 128 : 256, MINB) k_adjoint(Params P, StepArgs a) {
     extern __shared__ float4 s_warp[];
     adjoint_particle<D, P2GT, G2PT, FUSE, FUSE_V, EXT, true, (MINB >= 3)>(
         P, a, blockIdx.x * blockDim.x + threadIdx.x, s_warp + (threadIdx.x >> 5) * warp_slots<D, G2PT>());
@@ -804,6 +820,12 @@ static cudaError_t forward_d(bool g2p, bool p2g, bool all, const Params& P, cons
                 const size_t smem_agg = warps * warp_slots<D, true, true>() * sizeof(float4);
                 if (all) return go(k_forward<D, true, true, true, FUSE, false, true>, smem_agg);
                 return go(k_forward<D, true, true, false, FUSE, false, true>, smem_agg);
+            }
+        }
+        if constexpr (D == 3 && !FUSE) {
+            if (P.n_total <= P.wave) {
+                if (all) return go(k_forward<D, true, true, true, FUSE, false, true, kMinBlocksOneWave>, smem_p2g);
+                return go(k_forward<D, true, true, false, FUSE, false, true, kMinBlocksOneWave>, smem_p2g);
             }
         }
         if (all) return go(k_forward<D, true, true, true, FUSE, false>, smem_p2g);
@@ -847,9 +869,12 @@ static cudaError_t adjoint_d(bool p2gt, bool g2pt, const Params& P, const StepAr
         if constexpr (D == 2) {
             if (P.adj_blocks == 4) return go(k_adjoint<D, true, true, FUSE, FUSE_V, 4, false>, sm_g2pt);
         }
-        if (P.adj_blocks >= 3)
-            return go(k_adjoint<D, true, true, FUSE, FUSE_V, 3, false>, sm_g2pt);
-        return go(k_adjoint<D, true, true, FUSE, FUSE_V, 2, false>, sm_g2pt);
+        if (P.adj_blocks < 3 || (D == 3 && P.n_total <= P.wave))
+            return go(k_adjoint<D, true, true, FUSE, FUSE_V, kMinBlocksOneWave, false>, sm_g2pt);
+        if constexpr (D == 3) {
+            if (block <= 128) return go(k_adjoint<D, true, true, FUSE, FUSE_V, kBlocksOf128, false>, sm_g2pt);
+        }
+        return go(k_adjoint<D, true, true, FUSE, FUSE_V, 3, false>, sm_g2pt);
     }
     // the segment-edge halves run once per checkpoint segment
     if (p2gt) {
