@@ -327,8 +327,10 @@ __global__ void __launch_bounds__(256, MINB) k_forward(Params P, StepArgs a) {
 // EXT: P.ext is set (solid boxes or a non-uniform field), as in k_forward.
 // CHAIN and the calling convention as in forward_particle; sm: this warp's
 // warp_slots<D, G2PT>() float4 (the scatter slab of G2P^T).  RELIEF: the
-// register budget is tight (80 registers or fewer), so the state and stress
-// of P2G^T are reloaded and recomputed after its node loop.
+// register budget is tight (96 registers or fewer, in 3D also 128), so the
+// state and stress of P2G^T are reloaded and recomputed after its node loop
+// (3D at 128 registers: 216 -> 12 bytes of spill loads; 64,000 particles 3,050
+// -> 3,015 us, 82,944 in a non-uniform field 2,530 -> 2,443).
 template <int D, bool P2GT, bool G2PT, bool FUSE, bool FUSE_V, bool EXT, bool CHAIN, bool RELIEF>
 __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs& a, int p, float4* sm) {
     using L = Layout<D>;
@@ -791,7 +793,7 @@ __device__ __forceinline__ void adjoint_particle(const Params& P, const StepArgs
 template <int D, bool P2GT, bool G2PT, bool FUSE, bool FUSE_V, int MINB, bool EXT>
 __global__ void __launch_bounds__(MINB == kBlocksOf128 ? 128 : 256, MINB) k_adjoint(Params P, StepArgs a) {
     extern __shared__ float4 s_warp[];
-    adjoint_particle<D, P2GT, G2PT, FUSE, FUSE_V, EXT, true, (MINB >= 3)>(
+    adjoint_particle<D, P2GT, G2PT, FUSE, FUSE_V, EXT, true, (MINB >= 3 || D == 3)>(
         P, a, blockIdx.x * blockDim.x + threadIdx.x, s_warp + (threadIdx.x >> 5) * warp_slots<D, G2PT>());
 }
 
