@@ -231,56 +231,11 @@ __device__ __forceinline__ bool make_stencil(const float (&x)[D], const Params& 
     return ok;
 }
 
-template <int D>
-struct NodeTerm {
-    int node;        // node index within the instance grid (< 2^31 by configuration check)
-    int c[D];        // node coordinates
-    float w;         // weight N(x_p - x_i)
-    float gw[D];     // d w / d x_p
-    float dpos[D];   // x_i - x_p
-};
-
-template <int D>
-__device__ __forceinline__ void node_term(const Stencil<D>& s, int k, const Params& P, NodeTerm<D>& t) {
-    int o[D];
-    if (D == 2) {
-        o[0] = k / 3;
-        o[D - 1] = k % 3;
-    } else {
-        o[0] = k / 9;
-        o[1 % D] = (k / 3) % 3;
-        o[D - 1] = k % 3;
-    }
-    float w = 1.0f;
-#pragma unroll
-    for (int a = 0; a < D; ++a) w *= s.w[a][o[a]];
-    t.w = w;
-    int idx = 0;
-#pragma unroll
-    for (int c = 0; c < D; ++c) {
-        float g = s.dw[c][o[c]] * P.inv_dx;
-#pragma unroll
-        for (int a = 0; a < D; ++a)
-            if (a != c) g *= s.w[a][o[a]];
-        t.gw[c] = g;
-        t.dpos[c] = ((float)o[c] - s.r[c]) * P.dx;
-        t.c[c] = s.base[c] + o[c];
-        idx = idx * P.res + t.c[c];
-    }
-    t.node = idx;
-}
-
 // offset along axis b of stencil node k (node k = (o0, o1[, o2]), last axis fastest);
 // a compile-time constant inside unrolled loops over k
 template <int D>
 __device__ __forceinline__ constexpr int stencil_offset(int k, int b) {
     return D == 2 ? (b == 0 ? k / 3 : k % 3) : (b == 0 ? k / 9 : (b == 1 ? (k / 3) % 3 : k % 3));
-}
-
-// a + o d for a stencil offset o in {0, 1, 2}: with o a compile-time
-// constant (unrolled stencil loops) this is no instruction, one add or one FMA.
-__device__ __forceinline__ float add_offset(float a, int o, float d) {
-    return o == 0 ? a : (o == 1 ? a + d : fmaf(2.0f, d, a));
 }
 
 // Index of the stencil's base node within the instance grid, and the offset
